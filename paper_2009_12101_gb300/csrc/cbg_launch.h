@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "cbg_batched.cuh"
+#include "cbg_cycle.cuh"
 #include "cbg_kernels.cuh"
 #include "cbg_stream.cuh"
 
@@ -29,6 +30,10 @@ template <int FMT> struct Launcher {
     // resident blocks per SM of the per-step SpMV kernels of this code format (the CSR
     // Arnoldi kernel with one and 32 lanes per row, and the sliced-ELL kernel): the least
     static int occupancy_spmv();
+    // one restart cycle in one cooperative launch, the own rows of the basis in shared
+    // memory (resident) or in L2
+    static void cycle(bool resident, int grid, size_t smem, cudaStream_t s, const CycleArgs& a);
+    static bool cycle_fits(bool resident, size_t smem);
     // batched persistent solve with thread-block clusters of `cluster` blocks
     static cudaError_t batched(int cluster, int grid, size_t smem, cudaStream_t s, const BatchArgs& a);
     static int batched_max_clusters(int cluster, size_t smem);

@@ -137,6 +137,48 @@ template <int FMT> int Launcher<FMT>::occupancy_spmv()
 
 namespace cbg {
 
+// dynamic shared memory a block of the cycle kernel may have (opted in once per process)
+template <int FMT, bool RES> static bool cycle_kernel_fits(size_t smem)
+{
+    static const size_t room = [] {
+        cudaFuncAttributes fa{};
+        if (cudaFuncGetAttributes(&fa, k_cycle<FMT, RES>) != cudaSuccess ||
+            cudaFuncSetAttribute(k_cycle<FMT, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 TMA_SMEM_OPTIN - (int)fa.sharedSizeBytes) != cudaSuccess) {
+            cudaGetLastError();
+            return (size_t)0;
+        }
+        return (size_t)TMA_SMEM_OPTIN - fa.sharedSizeBytes;
+    }();
+    return smem <= room;
+}
+
+template <int FMT, bool RES> static void cycle_kernel_run(int grid, size_t smem, cudaStream_t s, const CycleArgs& a)
+{
+    cudaLaunchConfig_t cfg{};          // cooperative: the blocks wait on one another
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(CY_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, k_cycle<FMT, RES>, a);
+}
+
+template <int FMT> void Launcher<FMT>::cycle(bool resident, int grid, size_t smem, cudaStream_t s, const CycleArgs& a)
+{
+    if (resident) cycle_kernel_run<FMT, true>(grid, smem, s, a);
+    else cycle_kernel_run<FMT, false>(grid, smem, s, a);
+}
+
+template <int FMT> bool Launcher<FMT>::cycle_fits(bool resident, size_t smem)
+{
+    return resident ? cycle_kernel_fits<FMT, true>(smem) : cycle_kernel_fits<FMT, false>(smem);
+}
+
 template <int FMT> static void batched_opt_in(size_t smem)
 {
     cudaFuncSetAttribute(k_batched<FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

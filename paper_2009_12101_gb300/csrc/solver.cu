@@ -87,6 +87,9 @@ struct Ops {
     int (*occ_dot)();
     int (*occ_axpy)();
     int (*occ_spmv)();
+    void (*cycle)(bool, int, size_t, cudaStream_t, const CycleArgs&);
+    bool (*cycle_fits)(bool, size_t);
+    size_t (*cycle_smem)(int, int, int);
 };
 
 template <int F> Ops make_ops()
@@ -94,7 +97,8 @@ template <int F> Ops make_ops()
     return Ops{&Launcher<F>::dot, &Launcher<F>::axpy, &Launcher<F>::dot_tma,
                &Launcher<F>::tma_fits, &Launcher<F>::store, &Launcher<F>::spmv_code, &Launcher<F>::spmv_sell,
                &Launcher<F>::encode, &Launcher<F>::decode, &Launcher<F>::occupancy_dot,
-               &Launcher<F>::occupancy_axpy, &Launcher<F>::occupancy_spmv};
+               &Launcher<F>::occupancy_axpy, &Launcher<F>::occupancy_spmv, &Launcher<F>::cycle,
+               &Launcher<F>::cycle_fits, &CycleGeom<F>::smem};
 }
 
 const Ops& ops_for(int fmt)
@@ -106,6 +110,7 @@ const Ops& ops_for(int fmt)
 
 long long round_up(long long a, long long b) { return (a + b - 1) / b * b; }
 
+constexpr int CNT_CYCLE = 8;                      // DevArrays::counters slot of the single-launch cycle
 constexpr long long SPMV_TUNE_MIN_ROWS = 65536;   // create times the SpMV schedules from here on
 
 // Next basis format of the adaptive ladder (options.adapt): e4m3 -> bf16 -> f32 -> f64,
@@ -311,6 +316,7 @@ __global__ void k_init_state(DevState* st, double bnorm, double target, double e
 __global__ void k_cycle_start(DevArrays d, long long maxit, int m)
 {
     if (threadIdx.x != 0) return;
+    d.counters[CNT_CYCLE] = 0u;            // the single-launch cycle's arrivals
     DevState* st = d.st;
     const double beta = st->beta;
     int run = beta > st->target && st->iters < maxit && isfinite(beta);
@@ -452,6 +458,11 @@ struct cbg_handle {
     int grid_tma = 0;         // bulk-copy pipelined basis kernels: one block per SM
     int fmt0 = 0;             // the handle's basis format (options.adapt may move up from it)
     bool use_tma = false;
+    // one launch per restart cycle (cbg_cycle.cuh); grid 0: the stepwise kernels
+    int cycle_grid = 0, cycle_rows = 0, cycle_mcols = 0, cycle_lanes = 1;
+    bool cycle_resident = false;
+    size_t cycle_smem = 0;
+    float2* cycle_part = nullptr;  // block partials, norms and coefficients of the single-launch cycle
     // sliced-ELL copy of the per-step operator (chunks of 32 rows), used when the
     // create-time timing finds it faster than the CSR SpMV
     int* sell_len = nullptr;
@@ -639,6 +650,8 @@ double spmv_bytes(const cbg_handle* h)
 double store_bytes(const cbg_handle* h) { return (double)h->n * (8.0 + (double)fmt_bytes(h->fmt)); }
 
 // ------------------------------------------------------------------ launches per step
+void plan_cycle(cbg_handle* h);
+
 // Basis format of the following cycles: code stride and the format-dependent grids.
 void set_format(cbg_handle* h, int fmt)
 {
@@ -649,6 +662,72 @@ void set_format(cbg_handle* h, int fmt)
     h->grid_dot = std::max(1, (int)std::min<long long>(h->ld / DOT_MIN_ROWS, (long long)sms * std::max(1, op.occ_dot())));
     const long long axpy_blocks = h->ld / ((long long)THREADS * (16 / fmt_bytes(fmt)));
     h->grid_axpy = std::max(1, (int)std::min<long long>(axpy_blocks, (long long)sms * std::max(1, op.occ_axpy())));
+    plan_cycle(h);
+}
+
+// Whether a restart cycle runs as one launch (cbg_cycle.cuh), and how.  Measured against the
+// stepwise kernels, whole solves at restart 100 (ms, stepwise -> one launch): 5-point 64^2
+// f64 18.6 -> 4.8, 7-point 31^3 f16 13.9 -> 4.6, 64^3 f32 23.6 -> 14.6, 27 per row at
+// 262144 rows f64 2.75 -> 2.64; beyond CYCLE_MAX_ROWS the stepwise basis kernels, which
+// keep more bytes in flight, take the lead (96^3 f64 123 -> 140).
+constexpr long long CYCLE_MAX_ROWS = 300000;
+constexpr int CYCLE_MIN_BLOCK_ROWS = 64;   // fewer blocks cost less in the barriers and sums
+                                           // than they save in the products (64^2: 32 rows
+                                           // 4.85 ms, 64 4.79, 128 5.02)
+void plan_cycle(cbg_handle* h)
+{
+    h->cycle_grid = 0;
+    if (!h->cycle_part) return;
+    const Ops& op = ops_for(h->fmt);
+    const int mcols = (int)round_up(h->m + 1, 32);
+    const int blocks = std::min(num_sms(), CY_MAXG);
+    const int rows = std::max(CYCLE_MIN_BLOCK_ROWS, (int)round_up((h->n + blocks - 1) / blocks, CY_ROWS));
+    for (int resident = 1; resident >= 0; resident--) {
+        const size_t smem = op.cycle_smem(rows, mcols, resident ? h->m + 1 : 0);
+        if (!op.cycle_fits(resident != 0, smem)) continue;
+        h->cycle_grid = (int)((h->n + rows - 1) / rows);
+        h->cycle_rows = rows;
+        h->cycle_mcols = mcols;
+        h->cycle_resident = resident != 0;
+        h->cycle_smem = smem;
+        // few rows per block: more lanes share a row of the SpMV
+        h->cycle_lanes = h->group;
+        while (h->cycle_lanes < 8 && (long long)rows * h->cycle_lanes * 2 <= CY_CT) h->cycle_lanes *= 2;
+        return;
+    }
+}
+
+void enqueue_cycle(cbg_handle* h)
+{
+    CycleArgs a{};
+    a.d = h->d;
+    a.V = h->V;
+    a.ldb = h->ldb;
+    a.n = h->n;
+    a.nrows = h->ld;
+    a.rows = h->cycle_rows;
+    a.mcols = h->cycle_mcols;
+    a.rowptr = h->rowptr;
+    a.col = h->col;
+    a.valdf = h->valdf;
+    a.nnz = h->nnz;
+    if (h->opt.precond == CBG_PC_SPAI || h->opt.precond == CBG_PC_BJ4) {
+        a.prow = h->prow;
+        a.pcol = h->pcol;
+        a.pvals = h->pvals;
+        a.z = h->z;
+    }
+    a.lanes = h->cycle_lanes;
+    a.hexp = -h->pexp;
+    a.part = h->cycle_part;
+    a.norm = a.part + CY_PART;
+    a.coef = reinterpret_cast<double*>(a.norm + CY_NORM);
+    a.counter = h->d.counters + CNT_CYCLE;
+    a.fault = &h->d.st->fault;
+    a.limit = WAIT_LIMIT_CYCLES;
+    launch(h, 4, 0.0, [&] {
+        ops_for(h->fmt).cycle(h->cycle_resident, h->cycle_grid, h->cycle_smem, h->stream, a);
+    });
 }
 
 SellArgs sell_args(cbg_handle* h, const void* x, const double* xscale_dev, float* ydf, const int* active)
@@ -1046,7 +1125,10 @@ int run_solve(cbg_handle* h, const double* b, double* x, double tol, long long m
             cycles++;
             nvtxRangePushA("cbgmres cycle");
             enqueue_first_vector(h);
-            const int kcap = hs.kcap;
+            // (a requested stall of the pipelined dot needs the stepwise kernels)
+            const bool single = h->cycle_grid > 0 && h->test_stall == 0;
+            if (single) enqueue_cycle(h);
+            const int kcap = single ? 0 : hs.kcap;
             for (int j = 0; j < kcap; j++) {
                 if (j >= L) {
                     // keep at most L steps in flight; stop enqueueing once the cycle ended
@@ -1322,6 +1404,11 @@ int cbgmres_create(const cbg_csr* A, int restart, int fmt, const cbg_options* op
     size_t o_pn = take(sizeof(double) * (size_t)h->gridmax * 2);
     size_t o_ps = take(sizeof(double) * (size_t)h->gridmax * 2);
     size_t o_cnt = take(sizeof(unsigned int) * 16);
+    // one launch per restart cycle: the default arithmetic and orthogonalisation; profiling
+    // times the kernels of a step, so it keeps them apart
+    const bool single = o.arith == CBG_ARITH_DF32 && o.ortho == CBG_ORTHO_CGS && o.reorth == CBG_REORTH_ALWAYS &&
+                        h->valdf && !o.profile && n <= CYCLE_MAX_ROWS;
+    size_t o_cyc = single ? take(sizeof(float2) * (CY_PART + CY_NORM + CY_COEF)) : 0;
     unsigned char* blk = nullptr;
     TRY(dalloc(&blk, off));
     h->state_block = blk;
@@ -1341,6 +1428,7 @@ int cbgmres_create(const cbg_csr* A, int restart, int fmt, const cbg_options* op
     h->d.part_spmv = (double*)(blk + o_ps);
     h->d.counters = (unsigned int*)(blk + o_cnt);
     h->d.hist = nullptr;
+    if (single) h->cycle_part = (float2*)(blk + o_cyc);
     if (cudaHostAlloc((void**)&h->flag_host, sizeof(int), cudaHostAllocMapped) != cudaSuccess) TRY(CBG_ERR_CUDA);
     *h->flag_host = 0;
     if (cudaHostGetDevicePointer((void**)&h->flag_dev, h->flag_host, 0) != cudaSuccess) TRY(CBG_ERR_CUDA);
@@ -1453,6 +1541,7 @@ int cbgmres_create(const cbg_csr* A, int restart, int fmt, const cbg_options* op
             h->sell_chunks = 0;
         }
     }
+    plan_cycle(h);                        // (the SpMV's lanes are known now)
     if (o.profile) {
         const int pairs = 8 * restart + 64;
         h->prof_ev.resize(2 * pairs, nullptr);
