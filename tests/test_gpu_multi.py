@@ -43,6 +43,23 @@ def test_basis_dot_multi_matches_oracle(fmt, n, ncols, k):
     assert np.all(np.abs(H - ref) <= tol), np.max(np.abs(H - ref) / tol)
 
 
+@pytest.mark.parametrize("fmt", FORMATS)
+@pytest.mark.parametrize("n,ncols,k", [(4095, 15, 7), (4097, 16, 2), (8191, 17, 6), (300, 320, 3), (65537, 33, 1)])
+def test_basis_dot_multi_group_edges(fmt, n, ncols, k):
+    """Column groups of 16, pairs of vectors and row tiles at their edges, W with a leading
+    dimension beyond n (what lies there is not read)."""
+    torch, cb = need_gpu()
+    ld = (n + 4095) // 4096 * 4096
+    codes, scales, dec = _basis(fmt, n, ncols, ld, seed=n + 7 * ncols + k)
+    W = np.full((k, n + 5), np.nan)
+    W[:, :n] = np.random.default_rng(k).standard_normal((k, n))
+    H = cb.basis_dot_multi(fmt, n, torch.from_numpy(codes).cuda(), ld, scales, torch.from_numpy(W).cuda(),
+                           path="cuda").cpu().numpy()
+    ref = np.array([[O.dot(dec[c], np.ascontiguousarray(W[r, :n])) for r in range(k)] for c in range(ncols)])
+    tol = 1e-13 * np.linalg.norm(dec, axis=1)[:, None] * np.linalg.norm(W[:, :n], axis=1)[None, :]
+    assert np.all(np.abs(H - ref) <= tol), np.max(np.abs(H - ref) / tol)
+
+
 def test_basis_dot_multi_rejects_bad_arguments():
     torch, cb = need_gpu()
     V = torch.zeros((3, 4096 * 4), dtype=torch.uint8, device="cuda")
