@@ -569,6 +569,84 @@ void dfree(void* p)
     cudaFree(p);
 }
 
+// Device scratch of one call of a standalone entry point, as one block: take() lays the parts
+// out (256-byte aligned offsets), alloc() gets the block, at() turns an offset into its
+// address.  The block comes stream-ordered from a pool of the library's own on the current
+// device, which keeps up to POOL_KEEP bytes between calls and gives anything beyond back at
+// the next synchronisation (a cudaMalloc / cudaFree pair per part cost 0.5 ms of the 0.75 ms
+// of a projection of 2^20 x 200 e4m3, whose kernels take 0.23 ms).  The driver orders reuse
+// between streams and threads.  The debug build allocates with dalloc, for its guard tails.
+class Scratch {
+public:
+    explicit Scratch(cudaStream_t s) : s_(s) {}
+    ~Scratch()
+    {
+        if (!p_) return;
+#ifdef CBG_DEBUG
+        cudaStreamSynchronize(s_);
+        dfree(p_);
+#else
+        cudaFreeAsync(p_, s_);
+#endif
+    }
+    Scratch(const Scratch&) = delete;
+    Scratch& operator=(const Scratch&) = delete;
+    template <class T> T* take(size_t count)
+    {
+        const size_t o = bytes_;
+        bytes_ += (count * sizeof(T) + 255) / 256 * 256;
+        return reinterpret_cast<T*>(o);
+    }
+    int alloc()
+    {
+#ifdef CBG_DEBUG
+        return dalloc(&p_, bytes_);
+#else
+        cudaMemPool_t pool = nullptr;
+        const int rc = device_pool(&pool);
+        if (rc) return rc;
+        const cudaError_t e = cudaMallocFromPoolAsync((void**)&p_, bytes_, pool, s_);
+        if (e == cudaSuccess) return CBG_OK;
+        p_ = nullptr;
+        last_cuda_error = e;
+        return e == cudaErrorMemoryAllocation ? CBG_ERR_OOM : CBG_ERR_CUDA;
+#endif
+    }
+    template <class T> T* at(T* offset) const { return reinterpret_cast<T*>(p_ + reinterpret_cast<size_t>(offset)); }
+
+private:
+    static constexpr unsigned long long POOL_KEEP = 64ull << 20;
+    static int device_pool(cudaMemPool_t* out)
+    {
+        constexpr int NDEV = 64;
+        static std::mutex mu;
+        static cudaMemPool_t pools[NDEV] = {};           // per device, created on first use
+        int dev = 0;
+        CBG_CUDA(cudaGetDevice(&dev));
+        if (dev >= NDEV) {
+            CBG_CUDA(cudaDeviceGetDefaultMemPool(out, dev));
+            return CBG_OK;
+        }
+        std::lock_guard<std::mutex> lk(mu);
+        if (!pools[dev]) {
+            cudaMemPoolProps pr{};
+            pr.allocType = cudaMemAllocationTypePinned;
+            pr.location.type = cudaMemLocationTypeDevice;
+            pr.location.id = dev;
+            cudaMemPool_t p = nullptr;
+            unsigned long long keep = POOL_KEEP;
+            CBG_CUDA(cudaMemPoolCreate(&p, &pr));
+            CBG_CUDA(cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep));
+            pools[dev] = p;
+        }
+        *out = pools[dev];
+        return CBG_OK;
+    }
+    cudaStream_t s_;
+    unsigned char* p_ = nullptr;
+    size_t bytes_ = 0;
+};
+
 #ifdef CBG_DEBUG
 // CBG_OK when every live guard still holds its fill pattern
 int check_guards()
@@ -1794,45 +1872,46 @@ int cbg_basis_dot(int fmt, int arith, int64_t n, int ncols, const void* V, int64
     const bool tma = arith == CBG_ARITH_DF32;
     int grid = tma ? num_sms()
                    : (int)std::min<long long>(ld / DOT_MIN_ROWS, (long long)num_sms() * std::max(1, op.occ_dot()));
-    double *part = nullptr, *sc = nullptr, *out = nullptr, *wdf = nullptr;
-    unsigned int* cnt = nullptr;   // [0] last-block counter, [1] fault flag
-    int rc = dalloc(&part, (size_t)grid * MAXCOLS);
-    if (!rc) rc = dalloc(&sc, ncols);
-    if (!rc) rc = dalloc(&out, ncols);
-    if (!rc) rc = dalloc(&cnt, 2);
-    if (!rc && tma) rc = dalloc(&wdf, ld);
-    if (!rc) {
-        cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned int), s);
-        cudaMemcpyAsync(sc, scales, ncols * sizeof(double), cudaMemcpyHostToDevice, s);
-        DotArgs a{};
-        a.V = (const unsigned char*)V;
-        a.ldb = ld * fmt_bytes(fmt);
-        a.ncols = ncols;
-        a.scales = sc;
-        a.w = w;
-        a.nrows = ld;
-        a.part = part;
-        a.counter = cnt;
-        a.out = out;
-        if (tma) {
-            k_split_df<<<(int)std::min<long long>((ld + THREADS - 1) / THREADS, 4096), THREADS, 0, s>>>(
-                w, ld, reinterpret_cast<float*>(wdf));
-            a.wdf = reinterpret_cast<const float*>(wdf);
-            op.dot_tma(grid, s, a, reinterpret_cast<int*>(cnt + 1));
-        } else {
-            op.dot(arith, grid, s, a);
-        }
-        unsigned int flags[2] = {0u, 0u};
-        if (cudaGetLastError() != cudaSuccess ||
-            cudaMemcpyAsync(hout, out, ncols * sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaMemcpyAsync(flags, cnt, sizeof(flags), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess)
-            rc = CBG_ERR_CUDA;
-        else if (flags[1])
-            rc = CBG_ERR_TIMEOUT;
+    // one allocation: [barrier word, fault | h | scales | partials | split w]; the first two
+    // are read back together
+    Scratch sc(s);
+    unsigned int* cnt = sc.take<unsigned int>(4);
+    double* out = sc.take<double>(ncols);
+    double* scl = sc.take<double>(ncols);
+    double* part = sc.take<double>((size_t)grid * MAXCOLS);
+    double* wdf = sc.take<double>(tma ? ld : 0);
+    int rc = sc.alloc();
+    if (rc) return rc;
+    cnt = sc.at(cnt); out = sc.at(out); scl = sc.at(scl); part = sc.at(part); wdf = sc.at(wdf);
+    cudaMemsetAsync(cnt, 0, 4 * sizeof(unsigned int), s);
+    cudaMemcpyAsync(scl, scales, ncols * sizeof(double), cudaMemcpyHostToDevice, s);
+    DotArgs a{};
+    a.V = (const unsigned char*)V;
+    a.ldb = ld * fmt_bytes(fmt);
+    a.ncols = ncols;
+    a.scales = scl;
+    a.w = w;
+    a.nrows = ld;
+    a.part = part;
+    a.counter = cnt;
+    a.out = out;
+    if (tma) {
+        k_split_df<<<(int)std::min<long long>((ld + THREADS - 1) / THREADS, 4096), THREADS, 0, s>>>(
+            w, ld, reinterpret_cast<float*>(wdf));
+        a.wdf = reinterpret_cast<const float*>(wdf);
+        op.dot_tma(grid, s, a, reinterpret_cast<int*>(cnt + 1));
+    } else {
+        op.dot(arith, grid, s, a);
     }
-    dfree(part); dfree(sc); dfree(out); dfree(cnt); dfree(wdf);
-    return rc;
+    unsigned char host[256 + MAXCOLS * sizeof(double)];
+    const size_t at_out = (unsigned char*)out - (unsigned char*)cnt;
+    CBG_CUDA(cudaGetLastError());
+    CBG_CUDA(cudaMemcpyAsync(host, cnt, at_out + ncols * sizeof(double), cudaMemcpyDeviceToHost, s));
+    CBG_CUDA(cudaStreamSynchronize(s));
+    unsigned int flags[2];
+    std::memcpy(flags, host, sizeof(flags));
+    std::memcpy(hout, host + at_out, ncols * sizeof(double));
+    return flags[1] ? CBG_ERR_TIMEOUT : CBG_OK;
 }
 
 int cbg_basis_axpy(int fmt, int arith, int64_t n, int ncols, const void* V, int64_t ld, const double* scales,
@@ -1845,32 +1924,31 @@ int cbg_basis_axpy(int fmt, int arith, int64_t n, int ncols, const void* V, int6
     const Ops& op = ops_for(fmt);
     const long long blocks = ld / ((long long)THREADS * (16 / fmt_bytes(fmt)));
     int grid = (int)std::min<long long>(blocks, (long long)num_sms() * std::max(1, op.occ_axpy()));
-    double *sc = nullptr, *cf = nullptr, *pn = nullptr;
-    int rc = dalloc(&sc, ncols);
-    if (!rc) rc = dalloc(&cf, ncols);
-    if (!rc) rc = dalloc(&pn, (size_t)grid * 2);
-    if (!rc) {
-        cudaMemcpyAsync(sc, scales, ncols * sizeof(double), cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(cf, hcoef, ncols * sizeof(double), cudaMemcpyHostToDevice, s);
-        AxpyArgs a{};
-        a.V = (const unsigned char*)V;
-        a.ldb = ld * fmt_bytes(fmt);
-        a.ncols = ncols;
-        a.scales = sc;
-        a.coef = cf;
-        a.sign = -1.0;
-        a.w_in = w;
-        a.w_out = w;
-        a.nrows = ld;
-        a.n = n;
-        a.part_norm = pn;
-        op.axpy(arith, EPI_SUB, grid, s, a);
-        if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess) rc = CBG_ERR_CUDA;
-    }
-    dfree(sc); dfree(cf); dfree(pn);
-    return rc;
+    Scratch sc(s);
+    double* scl = sc.take<double>(ncols);
+    double* cf = sc.take<double>(ncols);
+    double* pn = sc.take<double>((size_t)grid * 2);
+    int rc = sc.alloc();
+    if (rc) return rc;
+    scl = sc.at(scl); cf = sc.at(cf); pn = sc.at(pn);
+    cudaMemcpyAsync(scl, scales, ncols * sizeof(double), cudaMemcpyHostToDevice, s);
+    cudaMemcpyAsync(cf, hcoef, ncols * sizeof(double), cudaMemcpyHostToDevice, s);
+    AxpyArgs a{};
+    a.V = (const unsigned char*)V;
+    a.ldb = ld * fmt_bytes(fmt);
+    a.ncols = ncols;
+    a.scales = scl;
+    a.coef = cf;
+    a.sign = -1.0;
+    a.w_in = w;
+    a.w_out = w;
+    a.nrows = ld;
+    a.n = n;
+    a.part_norm = pn;
+    op.axpy(arith, EPI_SUB, grid, s, a);
+    CBG_CUDA(cudaGetLastError());
+    CBG_CUDA(cudaStreamSynchronize(s));
+    return CBG_OK;
 }
-
-
 
 }  // extern "C"

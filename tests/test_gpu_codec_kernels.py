@@ -147,3 +147,39 @@ def test_decode_f32_special_values():
     nan = np.isnan(ref)
     assert np.array_equal(np.isnan(got), nan)
     assert np.array_equal(got[~nan].view(np.uint64), ref[~nan].view(np.uint64))
+
+
+def test_basis_products_from_threads_and_streams():
+    """The standalone products take their scratch from a pool shared by all callers: two
+    threads on their own streams get the bits of a single caller, for changing sizes."""
+    import threading
+    torch, cb = need_gpu()
+    rng = np.random.default_rng(11)
+    cases = []
+    for n, ncols in ((4096, 3), (300000, 40), (20000, 17)):
+        ld = (n + 4095) // 4096 * 4096
+        V = torch.zeros((ncols, ld), dtype=torch.float32, device="cuda")
+        V[:, :n] = torch.from_numpy(rng.standard_normal((ncols, n)).astype(np.float32)).cuda()
+        w = torch.zeros(ld, dtype=torch.float64, device="cuda")
+        w[:n] = torch.from_numpy(rng.standard_normal(n)).cuda()
+        h = cb.basis_dot("f32", "df32", n, V, ld, np.ones(ncols), w)
+        r = cb.basis_axpy("f32", "df32", n, V, ld, np.ones(ncols), h, w.clone())
+        cases.append((n, ld, V, w, ncols, h, r))
+    torch.cuda.synchronize()
+    bad = []
+
+    def work(k):
+        st = torch.cuda.Stream()
+        with torch.cuda.stream(st):
+            for i in range(30):
+                n, ld, V, w, ncols, h, r = cases[(i + k) % len(cases)]
+                x = w.clone()
+                g = cb.basis_dot("f32", "df32", n, V, ld, np.ones(ncols), x, stream=st)
+                cb.basis_axpy("f32", "df32", n, V, ld, np.ones(ncols), g, x, stream=st)
+                if not (np.array_equal(g, h) and torch.equal(x, r)):
+                    bad.append((k, i))
+
+    ts = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    [t.start() for t in ts]
+    [t.join() for t in ts]
+    assert not bad
