@@ -14,6 +14,7 @@
 #include <cstdio>
 #include <cstring>
 #include <fstream>
+#include <functional>
 #include <new>
 #include <numeric>
 #include <sstream>
@@ -86,6 +87,11 @@ struct cbg_batch {
     int *d_rowptr = nullptr, *d_col = nullptr;
     double *d_val = nullptr, *d_valp = nullptr, *d_dinv = nullptr;
     float* d_valpdf = nullptr;   // the per-step SpMV's values as FP32 hi / lo planes (or null)
+    long long* d_soff = nullptr; // ... and in sliced-ELL chunks of 32 rows (or null)
+    int* d_scol = nullptr;
+    float* d_sval = nullptr;
+    double* d_sval64 = nullptr;  // (f64 codes: FP64 values instead)
+    long long sell_entries = 0;
     unsigned char* d_V = nullptr;
     BatchOut* d_out = nullptr;
     unsigned int* d_queue = nullptr;
@@ -105,16 +111,20 @@ struct cbg_batch {
 
 namespace {
 
-size_t smem_bytes(const cbg_batch* bt, const Schedule& sc)
+// rows of w one block holds: a cluster share of the largest cooperative system, or a whole
+// small system (and the 16-entry tail the chunked loops read)
+long long block_rows(const cbg_batch* bt, const Schedule& sc)
 {
-    // rows of w one block holds: a cluster share of the largest cooperative system, or a
-    // whole small system
-    long long rows_cluster = sc.cluster > 1 ? ((bt->max_n + sc.cluster - 1) / sc.cluster + 15) / 16 * 16 : 0;
+    long long rows_cluster = sc.cluster > 1 ? ((bt->max_n + sc.cluster - 1) / sc.cluster + 31) / 32 * 32 : 0;
     long long rows_small = 0;
     for (const auto& s : bt->sys)
         if (sc.cluster == 1 || s.n < sc.split_rows) rows_small = std::max<long long>(rows_small, s.n);
-    long long rows = std::max(rows_cluster, rows_small);
-    return sizeof(BtSmem) + (size_t)(rows + 32) * sizeof(float2);
+    return (std::max(rows_cluster, rows_small) + 31) / 32 * 32 + 16;
+}
+
+size_t smem_bytes(const cbg_batch* bt, const Schedule& sc)
+{
+    return sizeof(BtSmem) + (size_t)block_rows(bt, sc) * 2 * sizeof(float);
 }
 
 // Per system: the power of two 2^s that brings the largest |value| of its per-step operator
@@ -146,11 +156,40 @@ void split_values_df(const double* v, long long n, int e, float* hi, float* lo)
     }
 }
 
+// The sliced-ELL copy of the packed values (the double-float planes into sval, or FP64 values
+// into sval64): a warp per chunk, chunk c belonging to the system csys[c]
+__global__ void k_batch_sell(const BatchSys* sys, const int* csys, long long nchunks, const int* rowptr,
+                             const int* col, const float* valdf, long long nnz, const double* val64, const long long* off,
+                             long long entries, int* scol, float* sval, double* sval64)
+{
+    const int lane = threadIdx.x & 31;
+    for (long long c = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; c < nchunks;
+         c += ((long long)gridDim.x * blockDim.x) >> 5) {
+        const BatchSys& s = sys[csys[c]];
+        const long long row = (c - s.ch_off) * 32 + lane;
+        const int* rp = rowptr + s.rp_off;
+        const int p0 = row < s.n ? rp[row] : 0, cnt = row < s.n ? rp[row + 1] - p0 : 0;
+        const int len = (int)((off[c + 1] - off[c]) >> 5);
+        for (int k = 0; k < len; k++) {
+            const long long q = off[c] + 32ll * k + lane, p = s.nz_off + p0 + k;
+            const bool in = k < cnt;
+            scol[q] = in ? col[p] : (row < s.n ? (int)row : 0);
+            if (sval64) {
+                sval64[q] = in ? val64[p] : 0.0;
+            } else {
+                sval[q] = in ? valdf[p] : 0.f;
+                sval[entries + q] = in ? valdf[nnz + p] : 0.f;
+            }
+        }
+    }
+}
+
 void free_batch(cbg_batch* bt)
 {
     if (!bt) return;
     cudaFree(bt->d_sys); cudaFree(bt->d_order); cudaFree(bt->d_rowptr); cudaFree(bt->d_col);
     cudaFree(bt->d_val); cudaFree(bt->d_valp); cudaFree(bt->d_dinv); cudaFree(bt->d_valpdf);
+    cudaFree(bt->d_soff); cudaFree(bt->d_scol); cudaFree(bt->d_sval); cudaFree(bt->d_sval64);
     cudaFree(bt->d_V); cudaFree(bt->d_out);
     cudaFree(bt->d_queue); cudaFree(bt->d_io);
     if (bt->h_io) cudaFreeHost(bt->h_io);
@@ -175,6 +214,11 @@ BatchArgs make_args(const cbg_batch* bt, const Schedule& sc, double tol, long lo
     a.dinv = bt->d_dinv;
     a.valpdf = bt->d_valpdf;
     a.nnz_all = bt->total_nnz;
+    a.sell_off = bt->d_soff;
+    a.sell_col = bt->d_scol;
+    a.sell_val = bt->d_sval;
+    a.sell_val64 = bt->d_sval64;
+    a.sell_entries = bt->sell_entries;
     a.io = bt->d_io;
     a.V = bt->d_V;
     a.out = bt->d_out;
@@ -183,7 +227,7 @@ BatchArgs make_args(const cbg_batch* bt, const Schedule& sc, double tol, long lo
     a.maxit = maxit;
     a.eps_bd = bt->opt.breakdown_eps;
     a.split_rows = sc.split_rows;
-    a.max_rows_block = 0;
+    a.max_rows_block = (int)block_rows(bt, sc);
     a.spmv_lanes = sc.lanes;
     return a;
 }
@@ -296,6 +340,56 @@ void cache_store(const char* path, const std::string& key, const Schedule& sc, d
     std::ofstream f(path, std::ios::app);
     f << "{\"key\": \"" << key << "\", \"cluster\": " << sc.cluster << ", \"split_rows\": " << sc.split_rows
       << ", \"lanes\": " << sc.lanes << ", \"ms\": " << ms << "}\n";
+}
+
+}  // namespace
+
+namespace {
+
+// Schedule without tuning: the cluster size and split threshold with the shortest simulated run
+// of the queue (systems in order of decreasing size, each taken by the first free cluster, the
+// ones below the threshold by the first free block).  A step of n rows on c blocks is taken as
+// 40,000 cycles of barriers, sums and scalar work (20,000 on one block) plus 43 cycles per row
+// of a block for 4-byte codes (measured with two blocks per SM; a little more for wider codes).
+// Measured against the fixed clusters of 8 from 8192 rows on, f32, 40 steps (ms): 96 systems of
+// 1024 .. 65,536 rows 8.6 -> 6.9, 120 up to 16,384 5.4 -> 3.4, 30 up to 4096 2.9 -> 1.1.
+Schedule default_schedule(const cbg_batch* bt)
+{
+    Schedule best;
+    double best_t = INFINITY;
+    const double per_row = 30.0 + 3.3 * fbytes(bt->fmt);
+    std::vector<double> free_at;
+    for (int c : {8, 4, 16, 2, 1})
+        for (int split : {1024, 2048, 4096, 8192, 16384}) {
+            const Schedule t{c, c > 1 ? split : (1 << 30)};
+            if (c == 1 && split > 1024) break;
+            const int grid = grid_for(bt, t, smem_bytes(bt, t));
+            if (grid <= 0) continue;
+            double makespan = 0.0;
+            // min-heap of the times at which clusters, later blocks, become free
+            free_at.assign(c > 1 ? grid / c : grid, 0.0);
+            bool blocks = c == 1;
+            auto later = std::greater<double>();
+            for (int i = 0; i < bt->nsys; i++) {
+                const int n = bt->sys[bt->order[i]].n;
+                if (!blocks && n < t.split_rows) {
+                    std::vector<double> per_block;
+                    for (double f : free_at) per_block.insert(per_block.end(), c, f);
+                    free_at.swap(per_block);
+                    std::make_heap(free_at.begin(), free_at.end(), later);
+                    blocks = true;
+                }
+                std::pop_heap(free_at.begin(), free_at.end(), later);
+                free_at.back() += blocks ? 2e4 + per_row * n : 4e4 + per_row * n / c;
+                makespan = std::max(makespan, free_at.back());
+                std::push_heap(free_at.begin(), free_at.end(), later);
+            }
+            if (makespan < best_t) {
+                best_t = makespan;
+                best = t;
+            }
+        }
+    return best;
 }
 
 }  // namespace
@@ -413,7 +507,42 @@ int cbgmres_create_batched(int nsys, const cbg_csr* As, int restart, int fmt, co
             rc = up((void**)&bt->d_valpdf, df.data(), df.size() * sizeof(float));
         }
     }
+    // sliced-ELL copy of those planes (f64: of the FP64 values), unless padding would add more than a quarter
+    std::vector<long long> soff;
+    std::vector<int> csys;
+    const bool sell_fmt = bt->d_valpdf || fmt == CBG_F64;
+    for (int i = 0; !rc && sell_fmt && i < nsys; i++) {
+        BatchSys& d = bt->sys[i];
+        const int* rp = rp_all.data() + d.rp_off;
+        d.ch_off = (long long)csys.size();
+        for (int r = 0; r < d.n; r += 32) {
+            int len = 0;
+            for (int q = r; q < std::min(r + 32, d.n); q++) len = std::max(len, rp[q + 1] - rp[q]);
+            soff.push_back(bt->sell_entries);
+            csys.push_back(i);
+            bt->sell_entries += 32ll * len;
+        }
+    }
+    soff.push_back(bt->sell_entries);
+    const bool sell = !rc && sell_fmt && bt->sell_entries <= bt->total_nnz + bt->total_nnz / 4;
     rc = rc ? rc : up((void**)&bt->d_sys, bt->sys.data(), bt->sys.size() * sizeof(BatchSys));
+    if (!rc && sell) {
+        int* d_csys = nullptr;
+        rc = up((void**)&d_csys, csys.data(), csys.size() * sizeof(int));
+        rc = rc ? rc : up((void**)&bt->d_soff, soff.data(), soff.size() * sizeof(long long));
+        if (!rc && (cudaMalloc((void**)&bt->d_scol, bt->sell_entries * sizeof(int)) != cudaSuccess ||
+                    cudaMalloc(fmt == CBG_F64 ? (void**)&bt->d_sval64 : (void**)&bt->d_sval,
+                               bt->sell_entries * sizeof(double)) != cudaSuccess))
+            rc = CBG_ERR_OOM;
+        if (!rc) {
+            const long long nch = (long long)csys.size();
+            k_batch_sell<<<(int)std::min<long long>((nch * 32 + 255) / 256, 4096), 256>>>(
+                bt->d_sys, d_csys, nch, bt->d_rowptr, bt->d_col, bt->d_valpdf, bt->total_nnz,
+                bt->d_valp ? bt->d_valp : bt->d_val, bt->d_soff, bt->sell_entries, bt->d_scol, bt->d_sval, bt->d_sval64);
+            if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(0) != cudaSuccess) rc = CBG_ERR_CUDA;
+        }
+        cudaFree(d_csys);
+    }
     if (!rc && cudaMalloc((void**)&bt->d_V, std::max<long long>(v_off, 256)) != cudaSuccess) rc = CBG_ERR_OOM;
     if (!rc && cudaMemset(bt->d_V, 0, std::max<long long>(v_off, 256)) != cudaSuccess) rc = CBG_ERR_CUDA;
     if (!rc && cudaMalloc((void**)&bt->d_out, nsys * sizeof(BatchOut)) != cudaSuccess) rc = CBG_ERR_OOM;
@@ -426,13 +555,7 @@ int cbgmres_create_batched(int nsys, const cbg_csr* As, int restart, int fmt, co
         free_batch(bt);
         return rc;
     }
-    // default schedule: the largest cluster this GPU co-schedules (up to 8); systems of
-    // 8192 rows or more on whole clusters
-    Schedule sc;
-    for (int c = 8; c >= 1; c /= 2) {
-        Schedule t{c, c > 1 ? 8192 : (1 << 30)};
-        if (grid_for(bt, t, smem_bytes(bt, t)) > 0) { sc = t; break; }
-    }
+    const Schedule sc = default_schedule(bt);
     bt->sched = sc;
     *out = bt;
     return CBG_OK;

@@ -9,12 +9,12 @@
 // block takes its own systems and runs alone.  No block ever spins on a flag: all waits
 // are __syncthreads or cluster barriers, which the hardware guarantees to complete.
 //
-// Per block, the block's rows of w live in shared memory as double-float pairs; only
+// Per block, the block's rows of w live in shared memory as FP32 hi and lo planes; only
 // the compressed basis, x and b are in HBM.
 #pragma once
 #include <cooperative_groups.h>
 
-#include "cbg_device.cuh"
+#include "cbg_kernels.cuh"
 
 namespace cbg {
 
@@ -31,6 +31,7 @@ struct BatchSys {
     long long nz_off;       // offset of its nonzeros (column indices are local)
     long long vec_off;      // offset of its b / x / dinv entries
     long long v_off;        // byte offset of its basis
+    long long ch_off;       // offset of its sliced-ELL chunks (BatchArgs::sell_off)
     double pscale;          // 2^s normalising its per-step operator (largest |value| in [1, 2))
     double hscale;          // 2^-s: Hessenberg columns back to the unscaled operator
 };
@@ -57,6 +58,16 @@ struct BatchArgs {
                             // [nnz_all] planes for the per-step SpMV in double-float, or null
                             // (FP64 products)
     long long nnz_all;
+    // the same planes in chunks of 32 rows (sliced ELL: entry k of the chunk's row l at
+    // sell_off[chunk] + 32 k + l, shorter rows padded with zero values), or null.  Read with one
+    // thread per row the CSR planes cost a cache line per lane and entry: most of the SM's
+    // cache is shared memory here, so the lines did not survive to the row's next entry
+    // (65,025 rows on 8 blocks, f32: 145,000 cycles per SpMV of 420,000 per step).
+    const long long* sell_off;
+    const int* sell_col;
+    const float* sell_val;  // hi [entries], lo [entries]; f64 codes: null, sell_val64 instead
+    const double* sell_val64;   // valp in the same order (FP64 products)
+    long long sell_entries;
     double* const* io;      // io[0] = b (packed), io[1] = x (packed); device table
     unsigned char* V;
     BatchOut* out;
@@ -65,7 +76,7 @@ struct BatchArgs {
     long long maxit;
     double eps_bd;
     int split_rows;
-    int max_rows_block;     // capacity of the shared-memory w (rows)
+    int max_rows_block;     // capacity of the shared-memory planes of w (rows, multiple of 16)
     int spmv_lanes;         // SpMV schedule: 1 = a thread per row (4 rows in flight), or 2, 4, 8
                             // lanes per row (the lanes split the row's nonzeros)
 };
@@ -77,10 +88,13 @@ struct BtSmem {
     double h[BT_MAXM + 1], u[BT_MAXM + 1], scale[BT_MAXM + 1];
     double red[BT_MAXM + 4];           // this block's partial sums (read by the cluster)
     double tot[BT_MAXM + 4];           // team totals
-    double wred[BT_THREADS / 32][BT_MAXM + 4];
+    double wred[BT_THREADS / 32][BT_MAXM + 4];   // (the dot: row splits' sums as float2)
+    double hn, inv, omega;             // of the current step (formed by one thread: an FP64 instruction
+    EncParams ep;                      // occupies the narrow pipe for a whole warp)
     int sys_idx;
     int stop;
-    float2 ws[1];                      // w rows of this block (max_rows_block + 16 entries)
+    alignas(16) float w[1];            // w of this block's rows: hi plane, then lo plane
+                                       // (max_rows_block entries each)
 };
 
 template <bool CLUSTER> struct Team {
@@ -138,6 +152,8 @@ __device__ __forceinline__ void block_sum(BtSmem* sm, const double (&v)[K], int 
 template <int FMT> struct BatchedSolver {
     static constexpr int BS = FmtInfo<FMT>::bytes;
     static constexpr int E = 16 / BS;
+    static constexpr int NW = BT_THREADS / 32;
+    static constexpr bool SCALED = FMT == I32 || FMT == I16 || FMT == BF16 || FMT == E4M3;   // encoding needs max |w|
 
     // ------------------------------------------------------------------ block kernels
     // w (own rows) = A_pc x  with x given by codes (column `col`, scaled) or FP64 array;
@@ -148,6 +164,7 @@ template <int FMT> struct BatchedSolver {
     {
         const int* rp = a.rowptr + s.rp_off;
         const int* ci = a.col + s.nz_off;
+        float* wl = sm->w + a.max_rows_block;
         const double* va = vals + s.nz_off;
         const double* bb = a.io[0] + s.vec_off;
         double ss = 0.0;
@@ -186,7 +203,8 @@ template <int FMT> struct BatchedSolver {
                     if (residual) v = __dsub_rn(bb[r], v);
                     float hi, lo;
                     split_f64(v, hi, lo);
-                    sm->ws[r - r0] = make_float2(hi, lo);
+                    sm->w[r - r0] = hi;
+                    wl[r - r0] = lo;
                     ss = __fma_rn(v, v, ss);
                 }
             }
@@ -205,6 +223,7 @@ template <int FMT> struct BatchedSolver {
     {
         const int* rp = a.rowptr + s.rp_off;
         const int* ci = a.col + s.nz_off;
+        float* wl = sm->w + a.max_rows_block;
         const float* vh = a.valpdf + s.nz_off;
         const float* vl = a.valpdf + a.nnz_all + s.nz_off;
         const bool xsplit = xscale != 1.0;                 // unit scale (float formats): no product
@@ -251,7 +270,8 @@ template <int FMT> struct BatchedSolver {
                         e = __fmaf_rn(lo, xsh, e);
                         two_sum(p, e, hi, lo);
                     }
-                    sm->ws[r - r0] = make_float2(hi, lo);
+                    sm->w[r - r0] = hi;
+                    wl[r - r0] = lo;
                     // w^2 = hi^2 + 2 hi lo to double-float accuracy
                     const float p = __fmul_rn(hi, hi);
                     float e = __fmaf_rn(hi, hi, -p);
@@ -266,6 +286,151 @@ template <int FMT> struct BatchedSolver {
         return df_to_double(ssS, ssC);
     }
 
+    // spmv_df on the sliced-ELL planes: a warp takes four chunks of 32 rows at a time (a lane
+    // per row), every load of columns and values is one contiguous 128-byte access, and the next
+    // entries are loaded while the current ones' gathers are in flight.
+    static __device__ double spmv_df_sell(const BatchArgs& a, const BatchSys& s, BtSmem* sm, int r0, int r1,
+                                          const void* x, double xscale)
+    {
+        constexpr int RW = 4;
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        float* wl = sm->w + a.max_rows_block;
+        const long long* off = a.sell_off + s.ch_off;
+        const float* vhp = a.sell_val;
+        const float* vlp = a.sell_val + a.sell_entries;
+        const bool xsplit = xscale != 1.0;
+        float xsh = 1.f, xsl = 0.f;
+        if (xsplit) split_f64(xscale, xsh, xsl);
+        float ssS = 0.f, ssC = 0.f;
+        const int cb = r0 >> 5, ce = (r1 + 31) >> 5;               // (r0 is a multiple of 32)
+        for (int c0 = cb + warp * RW; c0 < ce; c0 += NW * RW) {
+            float S[RW], C[RW], vh[RW], vl[RW];
+            long long p[RW];
+            int len[RW], c[RW], top = 0;
+#pragma unroll
+            for (int q = 0; q < RW; q++) {
+                const bool in = c0 + q < ce;
+                const long long b = in ? __ldg(off + c0 + q) : 0, e = in ? __ldg(off + c0 + q + 1) : 0;
+                p[q] = b + lane;
+                len[q] = (int)((e - b) >> 5);
+                top = max(top, len[q]);
+                S[q] = C[q] = 0.f;
+            }
+            auto entries = [&](int i) {                            // column -1: no entry
+#pragma unroll
+                for (int q = 0; q < RW; q++) {
+                    const bool in = i < len[q];
+                    vh[q] = in ? __ldg(vhp + p[q]) : 0.f;
+                    vl[q] = in ? __ldg(vlp + p[q]) : 0.f;
+                    c[q] = in ? __ldg(a.sell_col + p[q]) : -1;
+                    p[q] += 32;
+                }
+            };
+            entries(0);
+            for (int i = 0; i < top; i++) {
+                float xh[RW], xl[RW], fh[RW], fl[RW];
+#pragma unroll
+                for (int q = 0; q < RW; q++) {
+                    xh[q] = xl[q] = 0.f;
+                    fh[q] = vh[q];
+                    fl[q] = vl[q];
+                    if (c[q] >= 0) xval_df<FMT>(x, c[q], xh[q], xl[q]);
+                }
+                entries(i + 1);
+#pragma unroll
+                for (int q = 0; q < RW; q++) {
+                    if constexpr (SingleFloat<FMT>::value) df_mac(S[q], C[q], xh[q], fh[q], fl[q]);
+                    else df_mac2(S[q], C[q], xh[q], xl[q], fh[q], fl[q]);
+                }
+            }
+#pragma unroll
+            for (int q = 0; q < RW; q++) {
+                const int r = (c0 + q) * 32 + lane;
+                if (r < r1 && c0 + q < ce) {
+                    float hi, lo;
+                    two_sum(S[q], C[q], hi, lo);                   // renormalise
+                    if (xsplit) {
+                        const float pr = __fmul_rn(hi, xsh);
+                        float e = __fmaf_rn(hi, xsh, -pr);
+                        e = __fmaf_rn(hi, xsl, e);
+                        e = __fmaf_rn(lo, xsh, e);
+                        two_sum(pr, e, hi, lo);
+                    }
+                    sm->w[r - r0] = hi;
+                    wl[r - r0] = lo;
+                    const float pr = __fmul_rn(hi, hi);
+                    float e = __fmaf_rn(hi, hi, -pr);
+                    e = __fmaf_rn(__fadd_rn(hi, hi), lo, e);
+                    float t, te;
+                    two_sum(ssS, pr, t, te);
+                    ssC = __fadd_rn(ssC, __fadd_rn(te, e));
+                    ssS = t;
+                }
+            }
+        }
+        return df_to_double(ssS, ssC);
+    }
+
+    // the same for f64 codes, which keep FP64 products
+    static __device__ double spmv_sell64(const BatchArgs& a, const BatchSys& s, BtSmem* sm, int r0, int r1,
+                                         const double* x, double xscale)
+    {
+        constexpr int RW = 4;
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        float* wl = sm->w + a.max_rows_block;
+        const long long* off = a.sell_off + s.ch_off;
+        double ss = 0.0;
+        const int cb = r0 >> 5, ce = (r1 + 31) >> 5;
+        for (int c0 = cb + warp * RW; c0 < ce; c0 += NW * RW) {
+            double t[RW], v[RW];
+            long long p[RW];
+            int len[RW], c[RW], top = 0;
+#pragma unroll
+            for (int q = 0; q < RW; q++) {
+                const bool in = c0 + q < ce;
+                const long long b = in ? __ldg(off + c0 + q) : 0, e = in ? __ldg(off + c0 + q + 1) : 0;
+                p[q] = b + lane;
+                len[q] = (int)((e - b) >> 5);
+                top = max(top, len[q]);
+                t[q] = 0.0;
+            }
+            auto entries = [&](int i) {
+#pragma unroll
+                for (int q = 0; q < RW; q++) {
+                    const bool in = i < len[q];
+                    v[q] = in ? __ldg(a.sell_val64 + p[q]) : 0.0;
+                    c[q] = in ? __ldg(a.sell_col + p[q]) : -1;
+                    p[q] += 32;
+                }
+            };
+            entries(0);
+            for (int i = 0; i < top; i++) {
+                double xv[RW], f[RW];
+#pragma unroll
+                for (int q = 0; q < RW; q++) {
+                    f[q] = v[q];
+                    xv[q] = c[q] >= 0 ? x[c[q]] : 0.0;
+                }
+                entries(i + 1);
+#pragma unroll
+                for (int q = 0; q < RW; q++) t[q] = __fma_rn(f[q], xv[q], t[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < RW; q++) {
+                const int r = (c0 + q) * 32 + lane;
+                if (r < r1 && c0 + q < ce) {
+                    const double y = __dmul_rn(t[q], xscale);
+                    float hi, lo;
+                    split_f64(y, hi, lo);
+                    sm->w[r - r0] = hi;
+                    wl[r - r0] = lo;
+                    ss = __fma_rn(y, y, ss);
+                }
+            }
+        }
+        return ss;
+    }
+
     // The SpMVs above with L = a.spmv_lanes lanes per row (L = 2, 4, 8): the lanes of a
     // group take every L-th nonzero of the row and their partial sums meet in shuffles.
     // Groups walk the block's rows in warp-uniform passes, so every shuffle has the whole
@@ -276,6 +441,7 @@ template <int FMT> struct BatchedSolver {
     {
         const int* rp = a.rowptr + s.rp_off;
         const int* ci = a.col + s.nz_off;
+        float* wl = sm->w + a.max_rows_block;
         const double* va = vals + s.nz_off;
         const double* bb = a.io[0] + s.vec_off;
         const int L = a.spmv_lanes, lg = threadIdx.x & (L - 1), gpw = 32 / L;
@@ -301,7 +467,8 @@ template <int FMT> struct BatchedSolver {
                 if (residual) v = __dsub_rn(bb[r], v);
                 float hi, lo;
                 split_f64(v, hi, lo);
-                sm->ws[r - r0] = make_float2(hi, lo);
+                sm->w[r - r0] = hi;
+                    wl[r - r0] = lo;
                 ss = __fma_rn(v, v, ss);
             }
         }
@@ -313,6 +480,7 @@ template <int FMT> struct BatchedSolver {
     {
         const int* rp = a.rowptr + s.rp_off;
         const int* ci = a.col + s.nz_off;
+        float* wl = sm->w + a.max_rows_block;
         const float* vh = a.valpdf + s.nz_off;
         const float* vl = a.valpdf + a.nnz_all + s.nz_off;
         const bool xsplit = xscale != 1.0;
@@ -348,7 +516,8 @@ template <int FMT> struct BatchedSolver {
                     e = __fmaf_rn(lo, xsh, e);
                     two_sum(p, e, hi, lo);
                 }
-                sm->ws[r - r0] = make_float2(hi, lo);
+                sm->w[r - r0] = hi;
+                    wl[r - r0] = lo;
                 const float p = __fmul_rn(hi, hi);
                 float e = __fmaf_rn(hi, hi, -p);
                 e = __fmaf_rn(__fadd_rn(hi, hi), lo, e);
@@ -361,109 +530,226 @@ template <int FMT> struct BatchedSolver {
         return df_to_double(ssS, ssC);
     }
 
-    // partial h_k = sum over own rows of dec(V_k) w, k < ncols, into sm->red[0..ncols)
-    // (scale applied); one warp per column, lanes walk the rows in 16-byte chunks.
+    // partial h_k = sum over own rows of dec(V_k) w, k < ncols, into sm->red[0..ncols) (scale
+    // applied).  Warps are dealt out as row splits x groups of eight columns so that the
+    // slowest has the fewest (group, segment of 32 chunks) items; a warp reads its rows of w
+    // once for the eight columns (one column per warp read them from shared memory per
+    // column, with bank conflicts, and left warps idle while the basis was short).  Halves of
+    // a group are software-pipelined.
     static __device__ void dot(const BatchArgs& a, const BatchSys& s, BtSmem* sm, int r0, int r1, int ncols)
     {
+        constexpr int CG = 8, H = CG / 2;
+        static_assert(NW == 8, "the deal below assumes eight warps");
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        const unsigned char* Vs = a.V + s.v_off;
-        const int nloc = r1 - r0;
-        constexpr int U = 8;                               // 16-byte loads in flight per lane
-        for (int k = warp; k < ncols; k += BT_THREADS / 32) {
-            const unsigned char* cp = Vs + ((long long)k * s.ld + r0) * BS;
-            float S = 0.f, C = 0.f;
-            for (int b0 = lane * E; b0 < nloc; b0 += U * 32 * E) {
-                uint4 raw[U];
+        const long long vstride = (long long)s.ld * BS;
+        const unsigned char* vs = a.V + s.v_off + (long long)r0 * BS;
+        const int nch = (r1 - r0 + E - 1) / E, nseg = (nch + 31) >> 5, ngroups = (ncols + CG - 1) / CG;
+        const float* wl = sm->w + a.max_rows_block;
+        float2* red = reinterpret_cast<float2*>(&sm->wred[0][0]);
+        constexpr int RS = BT_MAXM + 4;
+        int lc = 0, best = 0x7fffffff;
 #pragma unroll
-                for (int q = 0; q < U; q++) {
-                    const int e0 = b0 + q * 32 * E;
-                    raw[q] = e0 < nloc ? ldg_stream(cp + (long long)e0 * BS) : make_uint4(0u, 0u, 0u, 0u);
+        for (int c = 0; c <= 3; c++) {                         // 2^c column groups at a time
+            const int items = ((ngroups + (1 << c) - 1) >> c) * ((nseg + (NW >> c) - 1) >> (3 - c));
+            if (items <= best) {
+                best = items;
+                lc = c;
+            }
+        }
+        const int wc = 1 << lc, lr = 3 - lc, wr = 1 << lr, mc = warp >> lr, mr = warp & (wr - 1);
+        for (int g = mc; g < ngroups; g += wc) {
+            const int c0 = g * CG, nc = ncols - c0 < CG ? ncols - c0 : CG;
+            float2 S2[CG / 2], C2[CG / 2];
+#pragma unroll
+            for (int q = 0; q < CG / 2; q++) { S2[q] = make_float2(0.f, 0.f); C2[q] = make_float2(0.f, 0.f); }
+            const unsigned char* vc = vs + (long long)c0 * vstride;
+            auto fetch = [&](int ch, int q0, uint4 (&raw)[H]) {
+                const unsigned char* p = vc + (long long)q0 * vstride + ch * 16;
+#pragma unroll
+                for (int q = 0; q < H; q++) {
+                    raw[q] = ch < nch && q0 + q < nc ? ldg_stream(p) : make_uint4(0u, 0u, 0u, 0u);
+                    p += vstride;
                 }
+            };
+            int ch = mr * 32 + lane;
+            uint4 ra[H], rb[H];
+            fetch(ch, 0, ra);
+            for (int sg = mr; sg < nseg; sg += wr) {
+                const int r = ch < nch ? ch * E : 0;
+                fetch(ch, H, rb);
+                float xh[E], xl[E];
 #pragma unroll
-                for (int q = 0; q < U; q++) {
-                    const int e0 = b0 + q * 32 * E;
-                    if (e0 >= nloc) break;
-                    Chunk<FMT> ch;
-                    decode_chunk<FMT>(raw[q], ch);
+                for (int e = 0; e < E; e += 2) {
+                    const float2 h2 = *reinterpret_cast<const float2*>(sm->w + r + e);
+                    const float2 l2 = *reinterpret_cast<const float2*>(wl + r + e);
+                    xh[e] = h2.x; xh[e + 1] = h2.y; xl[e] = l2.x; xl[e + 1] = l2.y;
+                }
+                auto accumulate = [&](const uint4& u0, const uint4& u1, float2& S, float2& C) {
+                    Chunk<FMT> k0, k1;
+                    decode_chunk<FMT>(u0, k0);
+                    decode_chunk<FMT>(u1, k1);
 #pragma unroll
                     for (int e = 0; e < E; e++) {
-                        const float2 wv = sm->ws[e0 + e];      // zero beyond nloc
-                        if constexpr (SingleFloat<FMT>::value) df_mac(S, C, ch.vh[e], wv.x, wv.y);
-                        else df_mac2(S, C, ch.vh[e], ch.vl[e], wv.x, wv.y);
+                        const float2 w2 = make_float2(xh[e], xh[e]), nw2 = make_float2(-xh[e], -xh[e]);
+                        const float2 l2 = make_float2(xl[e], xl[e]);
+                        if constexpr (SingleFloat<FMT>::value)
+                            df2_mac(S, C, make_float2(k0.vh[e], k1.vh[e]), w2, nw2, l2);
+                        else
+                            df2_mac2(S, C, make_float2(k0.vh[e], k1.vh[e]), make_float2(k0.vl[e], k1.vl[e]), w2, nw2, l2);
                     }
-                    df_renorm(S, C);
-                }
-            }
+                    df2_renorm(S, C);
+                };
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                const float oS = __shfl_xor_sync(0xFFFFFFFFu, S, o);
-                const float oC = __shfl_xor_sync(0xFFFFFFFFu, C, o);
-                df_add(S, C, oS, oC);
+                for (int q = 0; q < H; q += 2)
+                    if (q < nc) accumulate(ra[q], ra[q + 1], S2[q / 2], C2[q / 2]);
+                ch += wr * 32;
+                fetch(ch, 0, ra);
+#pragma unroll
+                for (int q = 0; q < H; q += 2)
+                    if (H + q < nc) accumulate(rb[q], rb[q + 1], S2[(H + q) / 2], C2[(H + q) / 2]);
             }
-            if (lane == 0) sm->red[k] = __dmul_rn(df_to_double(S, C), sm->scale[k]);
+            float S[CG], C[CG];
+#pragma unroll
+            for (int q = 0; q < CG / 2; q++) {
+                S[2 * q] = S2[q].x; S[2 * q + 1] = S2[q].y;
+                C[2 * q] = C2[q].x; C[2 * q + 1] = C2[q].y;
+            }
+            const int col = df_warp_fold<CG>(S, C, lane);
+            if ((lane & fold_low<CG>()) == 0 && col < nc) red[mr * RS + c0 + col] = make_float2(S[0], C[0]);
+        }
+        __syncthreads();
+        for (int c = threadIdx.x; c < ncols; c += BT_THREADS) {
+            float2 t = red[c];
+            for (int k = 1; k < wr; k++) df_add(t.x, t.y, red[k * RS + c].x, red[k * RS + c].y);
+            sm->red[c] = __dmul_rn(df_to_double(t.x, t.y), sm->scale[c]);
         }
         __syncthreads();
     }
 
-    // ws -= V coef over own rows; with NORMS, also the thread's sum of squares and max |w|
-    // of the result (FP64 from the DF value; only the last pass of a step needs them).
+    // w -= V coef over own rows; with NORMS, also the block's sum of squares (double-float,
+    // into sm->red[0]) and, for the formats whose scale needs it, the maximum of |w| (into
+    // sm->red[1]).  Blocks with fewer row chunks than threads split the columns over the
+    // lanes of a warp; the column loads are software-pipelined.
     template <bool NORMS>
     static __device__ void axpy(const BatchArgs& a, const BatchSys& s, BtSmem* sm, int r0, int r1, int ncols,
-                                const double* coef, double& ss, double& mx)
+                                const double* coef)
     {
         __shared__ float2 cdf[BT_MAXM + 1];
+        __shared__ float2 wsum[NW], wmax[NW];
         for (int k = threadIdx.x; k < ncols; k += BT_THREADS) {
             float hi, lo;
             split_f64(-coef[k] * sm->scale[k], hi, lo);
             cdf[k] = make_float2(hi, lo);
         }
         __syncthreads();
-        const unsigned char* Vs = a.V + s.v_off;
-        const int nloc = r1 - r0;
-        ss = 0.0;
-        mx = 0.0;
-        for (int e0 = threadIdx.x * E; e0 < nloc; e0 += BT_THREADS * E) {
-            float S[E], C[E];
+        constexpr int U = 4;
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const int nloc = r1 - r0, nch = (nloc + E - 1) / E;
+        const long long vstride = (long long)s.ld * BS;
+        const unsigned char* vs = a.V + s.v_off + (long long)r0 * BS;
+        float* wl = sm->w + a.max_rows_block;
+        int lk = 0;                                            // 2^lk column splits
+        while (lk < 3 && (nch << (lk + 1)) <= BT_THREADS) lk++;
+        const int ks = 1 << lk, cpw = 32 >> lk, mk = lane >> (5 - lk), mch = lane & (cpw - 1);
+        float ssS = 0.f, ssC = 0.f;
+        float2 mx = make_float2(0.f, 0.f);
+        for (int base = warp * cpw; base < nch; base += NW * cpw) {
+            const int ch = base + mch;
+            const bool in = ch < nch;
+            float2 S2[E / 2], C2[E / 2];
 #pragma unroll
-            for (int e = 0; e < E; e++) { S[e] = sm->ws[e0 + e].x; C[e] = sm->ws[e0 + e].y; }
-            const unsigned char* base = Vs + ((long long)r0 + e0) * BS;
-            constexpr int U = E <= 8 ? 8 : 4;                // columns in flight per thread
-            for (int k0 = 0; k0 < ncols; k0 += U) {
-                uint4 raw[U];
-#pragma unroll
-                for (int q = 0; q < U; q++)
-                    raw[q] = k0 + q < ncols ? ldg_stream(base + (long long)(k0 + q) * s.ld * BS)
-                                            : make_uint4(0u, 0u, 0u, 0u);
+            for (int e = 0; e < E / 2; e++) { S2[e] = make_float2(0.f, 0.f); C2[e] = make_float2(0.f, 0.f); }
+            const unsigned char* cp = vs + (long long)ch * 16;
+            auto fetch = [&](int k0, uint4 (&raw)[U]) {
+                const unsigned char* p = cp + (long long)k0 * vstride;
 #pragma unroll
                 for (int q = 0; q < U; q++) {
-                    if (k0 + q >= ncols) break;
-                    Chunk<FMT> ch;
-                    decode_chunk<FMT>(raw[q], ch);
-                    const float2 c = cdf[k0 + q];
+                    raw[q] = in && k0 + q * ks < ncols ? ldg_stream(p) : make_uint4(0u, 0u, 0u, 0u);
+                    p += ks * vstride;
+                }
+            };
+            // (a column past the last has zero codes and adds exact zeros)
+            auto accumulate = [&](int k0, const uint4 (&raw)[U]) {
 #pragma unroll
-                    for (int e = 0; e < E; e++) {
-                        if constexpr (SingleFloat<FMT>::value) df_mac(S[e], C[e], ch.vh[e], c.x, c.y);
-                        else df_mac2(S[e], C[e], ch.vh[e], ch.vl[e], c.x, c.y);
-                    }
-                    if ((q & 3) == 3) {
+                for (int q = 0; q < U; q++) {
+                    Chunk<FMT> cd;
+                    decode_chunk<FMT>(raw[q], cd);
+                    const float2 c = k0 + q * ks < ncols ? cdf[k0 + q * ks] : make_float2(0.f, 0.f);
+                    const float2 ch2 = make_float2(c.x, c.x), nch2 = make_float2(-c.x, -c.x), cl2 = make_float2(c.y, c.y);
 #pragma unroll
-                        for (int e = 0; e < E; e++) df_renorm(S[e], C[e]);
+                    for (int e = 0; e < E; e += 2) {
+                        if constexpr (SingleFloat<FMT>::value)
+                            df2_mac(S2[e / 2], C2[e / 2], make_float2(cd.vh[e], cd.vh[e + 1]), ch2, nch2, cl2);
+                        else
+                            df2_mac2(S2[e / 2], C2[e / 2], make_float2(cd.vh[e], cd.vh[e + 1]),
+                                     make_float2(cd.vl[e], cd.vl[e + 1]), ch2, nch2, cl2);
                     }
                 }
+#pragma unroll
+                for (int e = 0; e < E / 2; e++) df2_renorm(S2[e], C2[e]);
+            };
+            uint4 ra[U], rb[U];
+            fetch(mk, ra);
+            for (int k0 = mk; k0 - mk < ncols; k0 += 2 * U * ks) {   // (the same trips for every lane)
+                fetch(k0 + U * ks, rb);
+                accumulate(k0, ra);
+                if (k0 - mk + U * ks >= ncols) break;
+                fetch(k0 + 2 * U * ks, ra);
+                accumulate(k0 + U * ks, rb);
             }
 #pragma unroll
             for (int e = 0; e < E; e++) {
-                if (e0 + e < nloc) {
-                    df_renorm(S[e], C[e]);
-                    sm->ws[e0 + e] = make_float2(S[e], C[e]);
+                float S = e & 1 ? S2[e / 2].y : S2[e / 2].x, C = e & 1 ? C2[e / 2].y : C2[e / 2].x;
+                for (int o = cpw; o < 32; o <<= 1) {
+                    const float oS = __shfl_xor_sync(0xffffffffu, S, o), oC = __shfl_xor_sync(0xffffffffu, C, o);
+                    df_add(S, C, oS, oC);
+                }
+                const int r = ch * E + e;
+                if (in && mk == 0 && r < nloc) {
+                    df_add(S, C, sm->w[r], wl[r]);
+                    float h, l;
+                    two_sum(S, C, h, l);
+                    sm->w[r] = h;
+                    wl[r] = l;
                     if constexpr (NORMS) {
-                        const double d = df_to_double(S[e], C[e]);
-                        ss = __fma_rn(d, d, ss);
-                        // max |d| through the bit pattern (integer compare of non-negative doubles)
-                        const long long ab = __double_as_longlong(d) & 0x7FFFFFFFFFFFFFFFll;
-                        mx = ab > __double_as_longlong(mx) ? __longlong_as_double(ab) : mx;
+                        const float p = __fmul_rn(h, h);       // h^2 + 2 h l
+                        float q = __fmaf_rn(h, h, -p);
+                        q = __fmaf_rn(__fadd_rn(h, h), l, q);
+                        float t, te;
+                        two_sum(ssS, p, t, te);
+                        ssC = __fadd_rn(ssC, __fadd_rn(te, q));
+                        ssS = t;
+                        if constexpr (SCALED) {
+                            const float ah = fabsf(h), al = h < 0.f ? -l : l;
+                            if (!(ah < mx.x || (ah == mx.x && al <= mx.y))) mx = make_float2(ah, al);
+                        }
                     }
                 }
+            }
+        }
+        if constexpr (NORMS) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float oS = __shfl_xor_sync(0xffffffffu, ssS, o), oC = __shfl_xor_sync(0xffffffffu, ssC, o);
+                df_add(ssS, ssC, oS, oC);
+                if constexpr (SCALED) {
+                    const float h2 = __shfl_xor_sync(0xffffffffu, mx.x, o), l2 = __shfl_xor_sync(0xffffffffu, mx.y, o);
+                    if (!(h2 < mx.x || (h2 == mx.x && l2 <= mx.y))) mx = make_float2(h2, l2);
+                }
+            }
+            if (lane == 0) {
+                wsum[warp] = make_float2(ssS, ssC);
+                wmax[warp] = mx;
+            }
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                float2 t = wsum[0], m = wmax[0];
+                for (int w = 1; w < NW; w++) {
+                    df_add(t.x, t.y, wsum[w].x, wsum[w].y);
+                    if (!(wmax[w].x < m.x || (wmax[w].x == m.x && wmax[w].y <= m.y))) m = wmax[w];
+                }
+                sm->red[0] = df_to_double(t.x, t.y);
+                sm->red[1] = df_to_double(m.x, m.y);
             }
         }
         __syncthreads();
@@ -474,9 +760,72 @@ template <int FMT> struct BatchedSolver {
                                   double inv, const EncParams& ep)
     {
         unsigned char* dst = a.V + s.v_off + (long long)col * s.ld * BS;
-        for (int r = r0 + threadIdx.x; r < r1; r += BT_THREADS) {
-            const float2 wv = sm->ws[r - r0];
-            encode_store<FMT>(dst, r, __dmul_rn(df_to_double(wv.x, wv.y), inv), ep);
+        const float* wl = sm->w + a.max_rows_block;
+        for (int r = r0 + threadIdx.x; r < r1; r += BT_THREADS)
+            encode_store<FMT>(dst, r, __dmul_rn(df_to_double(sm->w[r - r0], wl[r - r0]), inv), ep);
+    }
+
+    // Warp 0: column j of the Hessenberg matrix (scaled back from the normalised operator,
+    // exactly), the previous rotations, the new one, g and the stopping tests.  The rotations
+    // form a first-order recurrence in the carried entry, evaluated as a warp scan of affine maps
+    // (as in the single-system store kernel) instead of a chain of j dependent steps.
+    static __device__ void givens(const BatchArgs& a, const BatchSys& s, BtSmem* sm, int j, int kcap, double target)
+    {
+        const int lane = threadIdx.x & 31, m = a.m;
+        double* Hc = sm->H + j * (m + 1);
+        const double hn = sqrt(sm->tot[0]), hnt = __dmul_rn(hn, s.hscale);
+        const int K = (j + 31) / 32, i0 = min(lane * K, j), i1 = min(i0 + K, j);   // K <= 2
+        double hv[3], A = 1.0, B = 0.0;                        // entries i0 .. i1 of the raw column
+#pragma unroll
+        for (int q = 0; q < 3; q++)
+            hv[q] = i0 + q <= j && q <= K ? __dmul_rn(__dadd_rn(sm->h[i0 + q], sm->u[i0 + q]), s.hscale) : 0.0;
+        const double h0 = __shfl_sync(0xffffffffu, hv[0], 0);
+        for (int i = i0; i < i1; i++) {
+            const double ai = -sm->sn[i], bi = __dmul_rn(sm->cs[i], i == i0 ? hv[1] : hv[2]);
+            B = __fma_rn(ai, B, bi);
+            A = __dmul_rn(ai, A);
+        }
+        double PA = A, PB = B;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double qa = __shfl_up_sync(0xffffffffu, PA, o), qb = __shfl_up_sync(0xffffffffu, PB, o);
+            if (lane >= o) {
+                PB = __fma_rn(PA, qb, PB);
+                PA = __dmul_rn(PA, qa);
+            }
+        }
+        double EA = __shfl_up_sync(0xffffffffu, PA, 1), EB = __shfl_up_sync(0xffffffffu, PB, 1);
+        if (lane == 0) { EA = 1.0; EB = 0.0; }
+        double x = __fma_rn(EA, h0, EB);                       // carried entry entering this lane's rotations
+        for (int i = i0; i < i1; i++) {
+            const double c = sm->cs[i], sn = sm->sn[i], h1 = i == i0 ? hv[1] : hv[2];
+            Hc[i] = __dadd_rn(__dmul_rn(c, x), __dmul_rn(sn, h1));
+            x = __dadd_rn(__dmul_rn(-sn, x), __dmul_rn(c, h1));
+        }
+        const double xl = __shfl_sync(0xffffffffu, x, j > 0 ? (j - 1) / K : 0);
+        if (lane == 0) {
+            const double r0v = j > 0 ? xl : h0;
+            const double rr = hypot(r0v, hnt);
+            double c = 1.0, sn = 0.0;
+            if (rr != 0.0) {
+                const double ri = 1.0 / rr;
+                c = __dmul_rn(r0v, ri);
+                sn = __dmul_rn(hnt, ri);
+            }
+            sm->cs[j] = c;
+            sm->sn[j] = sn;
+            Hc[j] = rr;
+            Hc[j + 1] = 0.0;
+            const double gj = sm->g[j];
+            sm->g[j + 1] = __dmul_rn(-sn, gj);
+            sm->g[j] = __dmul_rn(c, gj);
+            const double est = fabs(sm->g[j + 1]);
+            int stop = 0;
+            if (!isfinite(hnt) || !isfinite(sm->omega) || !isfinite(est)) stop = 3;
+            else if (!(hn > a.eps_bd * sm->omega)) stop = 2;   // both of the scaled operator
+            else if (est <= target) stop = 1;
+            else if (j + 1 >= kcap) stop = 4;
+            sm->stop = stop;
         }
     }
 
@@ -486,12 +835,13 @@ template <int FMT> struct BatchedSolver {
     {
         const BatchSys s = a.sys[si];
         const int m = a.m;
-        const int chunk = ((s.n + team.size - 1) / team.size + 15) / 16 * 16;
+        const int chunk = ((s.n + team.size - 1) / team.size + 31) / 32 * 32;   // whole sliced-ELL chunks
         const int r0 = min(s.n, team.rank * chunk);
         const int r1 = min(s.n, r0 + chunk);
         const int nloc = r1 - r0;
+        float* wl = sm->w + a.max_rows_block;
         // zero the w rows (and the 16-entry tail read by the chunked loops)
-        for (int i = threadIdx.x; i < nloc + 16; i += BT_THREADS) sm->ws[i] = make_float2(0.f, 0.f);
+        for (int i = threadIdx.x; i < nloc + 16; i += BT_THREADS) sm->w[i] = wl[i] = 0.f;
         double* x = a.io[1] + s.vec_off;
         const double* dinv = a.dinv ? a.dinv + s.vec_off : nullptr;
 
@@ -523,8 +873,7 @@ template <int FMT> struct BatchedSolver {
                 v[1] = 0.0;
                 double mxl = 0.0;
                 for (int r = r0 + threadIdx.x; r < r1; r += BT_THREADS) {
-                    const float2 wv = sm->ws[r - r0];
-                    mxl = fmax(mxl, fabs(df_to_double(wv.x, wv.y)));
+                    mxl = fmax(mxl, fabs(df_to_double(sm->w[r - r0], wl[r - r0])));
                 }
                 {
                     __syncthreads();
@@ -575,7 +924,10 @@ template <int FMT> struct BatchedSolver {
                     const double xs = __dmul_rn(sm->scale[j], s.pscale);
                     if (FMT != F64 && a.valpdf)                  // planes hold 2^s A_pc
                         om[0] = a.spmv_lanes > 1 ? spmv_df_lanes(a, s, sm, r0, r1, vj, sm->scale[j])
-                                                 : spmv_df(a, s, sm, r0, r1, vj, sm->scale[j]);
+                                : a.sell_off ? spmv_df_sell(a, s, sm, r0, r1, vj, sm->scale[j])
+                                             : spmv_df(a, s, sm, r0, r1, vj, sm->scale[j]);
+                    else if (FMT == F64 && a.spmv_lanes == 1 && a.sell_val64)
+                        om[0] = spmv_sell64(a, s, sm, r0, r1, reinterpret_cast<const double*>(vj), xs);
                     else
                         om[0] = a.spmv_lanes > 1 ? spmv_lanes<true>(a, s, sm, r0, r1, vj, xs, a.valp, false)
                                                  : spmv<true>(a, s, sm, r0, r1, vj, xs, a.valp, false);
@@ -583,74 +935,40 @@ template <int FMT> struct BatchedSolver {
                     block_sum<1>(sm, om, 1, j + 1);              // red[j+1] = omega^2 partial
                     dot(a, s, sm, r0, r1, j + 1);                // red[0..j]
                     team.reduce(sm, j + 2);
-                    const double omega = sqrt(sm->tot[j + 1]);
+                    if (threadIdx.x == BT_THREADS - 1) sm->omega = sqrt(sm->tot[j + 1]);
                     for (int i = threadIdx.x; i <= j; i += BT_THREADS) sm->h[i] = sm->tot[i];
                     __syncthreads();
-                    double ss, mx;
-                    axpy<false>(a, s, sm, r0, r1, j + 1, sm->h, ss, mx);   // (norms of w1 unused)
+                    axpy<false>(a, s, sm, r0, r1, j + 1, sm->h);           // (norms of w1 unused)
                     dot(a, s, sm, r0, r1, j + 1);
                     team.reduce(sm, j + 1);
                     for (int i = threadIdx.x; i <= j; i += BT_THREADS) sm->u[i] = sm->tot[i];
                     __syncthreads();
-                    axpy<true>(a, s, sm, r0, r1, j + 1, sm->u, ss, mx);
-                    double nv[1] = {ss};
-                    block_sum<1>(sm, nv, 1, 0);
-                    {   // block max of |w|
-                        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-                        double m2 = warp_max(mx);
-                        if (lane == 0) sm->wred[warp][1] = m2;
-                        __syncthreads();
-                        if (threadIdx.x == 0) {
-                            double mm = 0.0;
-                            for (int w = 0; w < BT_THREADS / 32; w++) mm = fmax(mm, sm->wred[w][1]);
-                            sm->red[1] = mm;
-                        }
-                    }
+                    axpy<true>(a, s, sm, r0, r1, j + 1, sm->u);
                     team.reduce(sm, 1);
-                    const double hn = sqrt(sm->tot[0]);
-                    double wmax = sm->red[1];
-                    if constexpr (CLUSTER) {
+                    if constexpr (CLUSTER && SCALED) {
                         cgx::cluster_group cl = cgx::this_cluster();
-                        for (int r = 0; r < team.size; r++) wmax = fmax(wmax, cl.map_shared_rank(sm->red, r)[1]);
+                        if (threadIdx.x == 0) {
+                            double wmax = sm->red[1];
+                            for (int r = 0; r < team.size; r++) wmax = fmax(wmax, cl.map_shared_rank(sm->red, r)[1]);
+                            sm->tot[1] = wmax;
+                        }
                         cl.sync();
                     }
-                    // Hessenberg column (scaled back from the normalised operator, exactly),
-                    // Givens rotations, stopping tests (identical in every block)
-                    if (threadIdx.x == 0) {
-                        double* Hc = sm->H + j * (m + 1);
-                        for (int i = 0; i <= j; i++) Hc[i] = __dmul_rn(__dadd_rn(sm->h[i], sm->u[i]), s.hscale);
-                        const double hnt = __dmul_rn(hn, s.hscale);
-                        Hc[j + 1] = hnt;
-                        double r0v = Hc[0];
-                        for (int i = 0; i < j; i++) {
-                            const double c = sm->cs[i], sn = sm->sn[i], r1v = Hc[i + 1];
-                            Hc[i] = __dadd_rn(__dmul_rn(c, r0v), __dmul_rn(sn, r1v));
-                            r0v = __dadd_rn(__dmul_rn(-sn, r0v), __dmul_rn(c, r1v));
-                        }
-                        const double rr = hypot(r0v, hnt);
-                        double c = 1.0, sn = 0.0;
-                        if (rr != 0.0) { c = r0v / rr; sn = hnt / rr; }
-                        sm->cs[j] = c;
-                        sm->sn[j] = sn;
-                        Hc[j] = rr;
-                        Hc[j + 1] = 0.0;
-                        const double gj = sm->g[j];
-                        sm->g[j + 1] = __dmul_rn(-sn, gj);
-                        sm->g[j] = __dmul_rn(c, gj);
-                        const double est = fabs(sm->g[j + 1]);
-                        int stop = 0;
-                        if (!isfinite(hnt) || !isfinite(omega) || !isfinite(est)) stop = 3;
-                        else if (!(hn > a.eps_bd * omega)) stop = 2;        // both of the scaled operator
-                        else if (est <= target) stop = 1;
-                        else if (j + 1 >= kcap) stop = 4;
-                        sm->stop = stop;
+                    // Hessenberg column, Givens rotations, stopping tests (warp 0) and what the
+                    // encoding needs (warp 1), identical in every block
+                    if (threadIdx.x < 32) {
+                        givens(a, s, sm, j, kcap, target);
+                    } else if (threadIdx.x == 32) {
+                        const double inv = 1.0 / sqrt(sm->tot[0]);
+                        sm->inv = inv;
+                        sm->ep = enc_params(FMT, SCALED ? __dmul_rn(CLUSTER ? sm->tot[1] : sm->red[1], inv) : 1.0);
                     }
                     __syncthreads();
                     iters++;
                     k = j + 1;
                     if (sm->stop) break;
-                    const double inv = 1.0 / hn;
-                    const EncParams ep = enc_params(FMT, __dmul_rn(wmax, inv));
+                    const double inv = sm->inv;
+                    const EncParams ep = sm->ep;
                     if (threadIdx.x == 0) sm->scale[j + 1] = ep.scale;
                     encode(a, s, sm, r0, r1, j + 1, inv, ep);
                 }
@@ -664,14 +982,15 @@ template <int FMT> struct BatchedSolver {
                     }
                 }
                 __syncthreads();
-                // x += D^{-1} V y over own rows
+                // x += D^{-1} V y over own rows (the scales folded into y: one FP64 FMA per element)
+                for (int i = threadIdx.x; i < k; i += BT_THREADS) sm->h[i] = __dmul_rn(sm->scale[i], sm->y[i]);
+                __syncthreads();
                 {
                     const unsigned char* Vs = a.V + s.v_off;
                     for (int r = r0 + threadIdx.x; r < r1; r += BT_THREADS) {
                         double t = 0.0;
                         for (int c2 = 0; c2 < k; c2++)
-                            t = __fma_rn(__dmul_rn(code_value<FMT>(Vs + (long long)c2 * s.ld * BS, r), sm->scale[c2]),
-                                         sm->y[c2], t);
+                            t = __fma_rn(code_value<FMT>(Vs + (long long)c2 * s.ld * BS, r), sm->h[c2], t);
                         if (dinv) t = __dmul_rn(dinv[r], t);
                         x[r] = __dadd_rn(x[r], t);
                     }
