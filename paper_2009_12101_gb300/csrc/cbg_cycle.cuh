@@ -129,16 +129,6 @@ __device__ __forceinline__ uint4 ld_cg16(const void* p)
     return __ldcg(reinterpret_cast<const uint4*>(p));
 }
 
-// (S, C) folded over the warp
-__device__ __forceinline__ void cy_warp_fold(float& S, float& C)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float s2 = __shfl_xor_sync(0xffffffffu, S, o), c2 = __shfl_xor_sync(0xffffffffu, C, o);
-        df_add(S, C, s2, c2);
-    }
-}
-
 // (S, C) += y^2 for a renormalised pair y = h + l
 __device__ __forceinline__ void cy_add_square(float& S, float& C, float h, float l)
 {
@@ -276,7 +266,7 @@ template <int FMT, bool RES> struct Cycle {
                 }
             }
         }
-        cy_warp_fold(ssS, ssC);
+        df_warp_sum(ssS, ssC);
         if ((threadIdx.x & 31) == 0) sm.wsum[threadIdx.x >> 5] = make_float2(ssS, ssC);
     }
 
@@ -571,7 +561,7 @@ template <int FMT, bool RES> struct Cycle {
             }
         }
         if constexpr (NORMS) {
-            cy_warp_fold(ssS, ssC);
+            df_warp_sum(ssS, ssC);
             fold_max(mx);
             if ((threadIdx.x & 31) == 0) {
                 sm.wsum[threadIdx.x >> 5] = make_float2(ssS, ssC);
@@ -622,7 +612,7 @@ template <int FMT, bool RES> struct Cycle {
                 df_add(s.x, s.y, v[u].x, v[u].y);
                 if (!(w[u].x < m.x || (w[u].x == m.x && w[u].y <= m.y))) m = w[u];
             }
-            cy_warp_fold(s.x, s.y);
+            df_warp_sum(s.x, s.y);
             fold_max(m);
             if (lane == 0) {
                 const double hn = sqrt(df_to_double(s.x, s.y)), inv = 1.0 / hn;

@@ -307,6 +307,22 @@ template <int FMT> __device__ __forceinline__ void decode_chunk(const uint4& raw
     }
 }
 
+// (S, C) += the chunk's rows times w (pairs of neighbouring rows; nw2 = -w2), renormalised
+template <int FMT>
+__device__ __forceinline__ void df2_mac_chunk(float2& S, float2& C, const Chunk<FMT>& ch, const float2* w2,
+                                              const float2* nw2, const float2* l2)
+{
+#pragma unroll
+    for (int e = 0; e < Chunk<FMT>::E; e += 2) {
+        if constexpr (SingleFloat<FMT>::value)
+            df2_mac(S, C, make_float2(ch.vh[e], ch.vh[e + 1]), w2[e / 2], nw2[e / 2], l2[e / 2]);
+        else
+            df2_mac2(S, C, make_float2(ch.vh[e], ch.vh[e + 1]), make_float2(ch.vl[e], ch.vl[e + 1]), w2[e / 2],
+                     nw2[e / 2], l2[e / 2]);
+    }
+    df2_renorm(S, C);
+}
+
 // Exact FP64 value of one code (scale not applied); used by the FP64 arithmetic mode,
 // the SpMV and the decode kernel.
 template <int FMT> __device__ __forceinline__ double code_value(const void* base, int64_t i)
@@ -437,6 +453,32 @@ __device__ __forceinline__ double warp_max(double v)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xFFFFFFFFu, v, o));
     return v;
+}
+
+// (S, C) summed over the warp in double-float (every lane holds the result)
+__device__ __forceinline__ void df_warp_sum(float& S, float& C)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float s2 = __shfl_xor_sync(0xFFFFFFFFu, S, o), c2 = __shfl_xor_sync(0xFFFFFFFFu, C, o);
+        df_add(S, C, s2, c2);
+    }
+}
+
+// The block's double-float sum of the threads' (S, C); valid in warp 0.  red: shared, one entry
+// per warp.  All threads call it.
+__device__ __forceinline__ float2 df_block_sum(float S, float C, float2* red)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    df_warp_sum(S, C);
+    if (lane == 0) red[warp] = make_float2(S, C);
+    __syncthreads();
+    float2 t = make_float2(0.f, 0.f);
+    if (warp == 0) {
+        if (lane < nw) t = red[lane];
+        df_warp_sum(t.x, t.y);
+    }
+    return t;
 }
 
 // maximum of non-negative doubles over the warp, compared as bit patterns with 32-bit

@@ -138,6 +138,26 @@ __device__ __forceinline__ void block_reduce_norm_parts(const double* part, int 
     block_sum_max(s, __hiloint2double((int)mh, (int)ml), rs, rm, ss, mx);
 }
 
+// The last block's ||.|| from per-block double-float sums of squares part[b] (all threads call
+// it; valid in thread 0): thread t adds the pairs t, t + blockDim.x, ..., then a fixed tree.
+__device__ __forceinline__ double df_block_norm(const float2* part, int np)
+{
+    __shared__ float2 red[32];
+    float S = 0.f, C = 0.f;
+    for (int p0 = threadIdx.x; p0 < np; p0 += 4 * blockDim.x) {
+        float2 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+            const int p = p0 + u * blockDim.x;
+            v[u] = p < np ? __ldcg(part + 2 * p) : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; u++) df_add(S, C, v[u].x, v[u].y);
+    }
+    const float2 t = df_block_sum(S, C, red);
+    return threadIdx.x == 0 ? sqrt(df_to_double(t.x, t.y)) : 0.0;
+}
+
 // The last block's sums over the per-block partials of nitems items: item i is
 // sum_{b < nb} part[b * ldp + i], handed to emit(i, sum) by lane 0 of the warp that
 // computed it.  Warp w of nwarps takes the items 2w, 2w + 1, then 2(w + nwarps), ...;
@@ -699,14 +719,51 @@ __global__ void __launch_bounds__(THREADS, FmtInfo<FMT>::bytes >= 8 ? 4 : (FmtIn
     }
     if constexpr (EPI == EPI_SUB) {
         if (!a.counter) return;
-        if constexpr (ARITH == ARITH_DF32) ss = df_to_double(ssS, ssC);
-        double s, m;
-        block_sum_max(ss, __hiloint2double((int)mxh, (int)mxl), red_s, red_m, s, m);
-        if (threadIdx.x == 0) {
-            a.part_norm[2 * blockIdx.x] = s;
-            a.part_norm[2 * blockIdx.x + 1] = m;
-        }
-        {
+        if constexpr (ARITH == ARITH_DF32) {
+            // sums in double-float (with the dot's and the SpMV's: 2 % of a large solve, which
+            // the FP64 trees of every block spent on the narrow pipe)
+            __shared__ float2 red_df[THREADS / 32];
+            const float2 t = df_block_sum(ssS, ssC, red_df);
+            const double m0 = warp_max_nonneg(__hiloint2double((int)mxh, (int)mxl));
+            if ((threadIdx.x & 31) == 0) red_m[threadIdx.x >> 5] = m0;
+            __syncthreads();
+            if (threadIdx.x < 32) {
+                const double m = warp_max_nonneg(threadIdx.x < THREADS / 32 ? red_m[threadIdx.x] : 0.0);
+                if (threadIdx.x == 0) {
+                    reinterpret_cast<float2*>(a.part_norm)[2 * blockIdx.x] = t;
+                    a.part_norm[2 * blockIdx.x + 1] = m;
+                }
+            }
+            if (last_block(a.counter)) {
+                const double wn = df_block_norm(reinterpret_cast<const float2*>(a.part_norm), gridDim.x);
+                unsigned int h = 0u, l = 0u;           // the maximum, on bit patterns
+                for (int p = threadIdx.x; p < gridDim.x; p += THREADS) {
+                    const double v = __ldcg(a.part_norm + 2 * p + 1);
+                    const unsigned int vh = (unsigned int)__double2hiint(v), vl = (unsigned int)__double2loint(v);
+                    if (vh > h || (vh == h && vl > l)) {
+                        h = vh;
+                        l = vl;
+                    }
+                }
+                const double m1 = warp_max_nonneg(__hiloint2double((int)h, (int)l));
+                if ((threadIdx.x & 31) == 0) red_m[threadIdx.x >> 5] = m1;
+                __syncthreads();
+                if (threadIdx.x < 32) {
+                    const double m = warp_max_nonneg(threadIdx.x < THREADS / 32 ? red_m[threadIdx.x] : 0.0);
+                    if (threadIdx.x == 0) {
+                        a.st->wnorm = wn;
+                        a.st->wmax = m;
+                        if (a.reorth_flag) *a.reorth_flag = wn < a.eta * a.st->omega ? 1 : 0;
+                    }
+                }
+            }
+        } else {
+            double s, m;
+            block_sum_max(ss, __hiloint2double((int)mxh, (int)mxl), red_s, red_m, s, m);
+            if (threadIdx.x == 0) {
+                a.part_norm[2 * blockIdx.x] = s;
+                a.part_norm[2 * blockIdx.x + 1] = m;
+            }
             if (last_block(a.counter)) {
                 double s2, m2;
                 block_reduce_norm_parts(a.part_norm, gridDim.x, s2, m2);
@@ -1095,7 +1152,16 @@ __global__ void __launch_bounds__(THREADS) k_spmv(SpmvArgs a)
     const double mx = __longlong_as_double((long long)mxb);
     if constexpr (MODE == SPMV_PLAIN || MODE == SPMV_ACCUM) return;
     else {
-        if (dfrows) ss = df_to_double(ssS, ssC);
+        if (dfrows) {                        // omega of the double-float rows, summed in double-float
+            __shared__ float2 red_df[THREADS / 32];
+            const float2 t = df_block_sum(ssS, ssC, red_df);
+            if (threadIdx.x == 0) reinterpret_cast<float2*>(a.part)[2 * blockIdx.x] = t;
+            if (last_block(a.counter)) {
+                const double om = df_block_norm(reinterpret_cast<const float2*>(a.part), gridDim.x);
+                if (threadIdx.x == 0) a.st->omega = om;
+            }
+            return;
+        }
         double s, m;
         block_sum_max(ss, mx, red_s, red_m, s, m);
         if (threadIdx.x == 0) {
@@ -1151,7 +1217,7 @@ template <int XFMT>
 __global__ void __launch_bounds__(THREADS) k_spmv_sell(SellArgs a)
 {
     if (a.active && *a.active == 0) return;
-    __shared__ double red_s[THREADS / 32], red_m[THREADS / 32];
+    __shared__ float2 red_df[THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr bool XEXACT = XFMT == F32 || XFMT == F16 || XFMT == BF16 || XFMT == E4M3 || XFMT == I16;
     const double xs = a.xscale_dev ? *a.xscale_dev : 1.0;
@@ -1223,16 +1289,11 @@ __global__ void __launch_bounds__(THREADS) k_spmv_sell(SellArgs a)
             dfadd(ssS, ssC, p, e);
         }
     }
-    double t, tm;
-    block_sum_max(df_to_double(ssS, ssC), 0.0, red_s, red_m, t, tm);
-    if (threadIdx.x == 0) {
-        a.part[2 * blockIdx.x] = t;
-        a.part[2 * blockIdx.x + 1] = 0.0;
-    }
+    const float2 t = df_block_sum(ssS, ssC, red_df);
+    if (threadIdx.x == 0) reinterpret_cast<float2*>(a.part)[2 * blockIdx.x] = t;
     if (last_block(a.counter)) {
-        double s2, m2;
-        block_reduce_norm_parts(a.part, gridDim.x, s2, m2);
-        if (threadIdx.x == 0) a.st->omega = sqrt(s2);
+        const double om = df_block_norm(reinterpret_cast<const float2*>(a.part), gridDim.x);
+        if (threadIdx.x == 0) a.st->omega = om;
     }
 }
 

@@ -64,30 +64,31 @@ __device__ __forceinline__ void record_fault(DevState* st, int* fault)
 // Barrier of all blocks of a cooperative launch on one counter word: bits 0..30 count the
 // arrivals, bit 31 is the sense, flipped by the last arrival (which also zeroes the
 // count), so the word is ready for the next launch as it is left.  Thread 0 of each
-// block arrives and waits (bounded: false when the wait gave up); the fences order the
-// block's writes before its arrival and the other blocks' writes before its departure.
+// block arrives (releasing the block's writes) and polls (acquiring the others'; bounded:
+// false when the wait gave up).
 __device__ __forceinline__ bool grid_barrier(unsigned int* cnt, long long limit)
 {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned sense = *(volatile unsigned*)cnt & 0x80000000u;
-        const unsigned old = atomicAdd(cnt, 1u);
+        unsigned sense, old, now;
+        asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(sense) : "l"(cnt) : "memory");
+        sense &= 0x80000000u;
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(old) : "l"(cnt) : "memory");
         int good = 1;
         if ((old & 0x7FFFFFFFu) == gridDim.x - 1) {
-            atomicExch(cnt, sense ^ 0x80000000u);
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(cnt), "r"(sense ^ 0x80000000u) : "memory");
         } else {
             const long long t0 = clock64();
-            while ((*(volatile unsigned*)cnt & 0x80000000u) == sense) {
+            for (;;) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(cnt) : "memory");
+                if ((now & 0x80000000u) != sense) break;
                 if (clock64() - t0 > limit) {
                     good = 0;
                     break;
                 }
-                __nanosleep(32);
             }
         }
-        __threadfence();
         ok = good;
     }
     __syncthreads();
@@ -169,8 +170,11 @@ __device__ __forceinline__ void tma_produce(unsigned char* ring, int stage_bytes
 
 // ============================================================== h = V^T w  (CGS)
 // Consumer warp of the dot: rows r .. r+E-1 of the tile and the CGW = CG/2 columns
-// starting at q0 within the stage, as packed pairs.  A missing column (>= nc) holds
-// stale codes; its lane of the pair is never read back (only columns < nc are kept).
+// starting at q0 within the stage.  The packed FP32x2 operations take two neighbouring rows
+// of one column: codes and w both lie so in registers as they are loaded (pairs of columns
+// need every code moved next to its partner's and w duplicated: a third more instructions, on
+// the pipes the products run on).  Component x of S2[q], C2[q] sums the even rows, y the odd
+// ones.  A missing column (>= nc) holds stale codes; its sums are never read back.
 template <int FMT, bool FULL>
 __device__ __forceinline__ void dot_consume(const unsigned char* st, int r, int q0, int nc, float2* S2, float2* C2)
 {
@@ -180,25 +184,19 @@ __device__ __forceinline__ void dot_consume(const unsigned char* st, int r, int 
     const float* wt = reinterpret_cast<const float*>(st + CG * G::COLB);
     load_floats<E>(wt + r, wh);
     load_floats<E>(wt + G::TILE + r, wl);
+    float2 w2[E / 2], nw2[E / 2], l2[E / 2];
 #pragma unroll
-    for (int q = 0; q < CGW; q += 2) {
+    for (int e = 0; e < E; e += 2) {
+        w2[e / 2] = make_float2(wh[e], wh[e + 1]);
+        nw2[e / 2] = make_float2(-wh[e], -wh[e + 1]);
+        l2[e / 2] = make_float2(wl[e], wl[e + 1]);
+    }
+#pragma unroll
+    for (int q = 0; q < CGW; q++) {
         if (!FULL && q0 + q >= nc) break;
-        const uint4 r0 = *reinterpret_cast<const uint4*>(st + (q0 + q) * G::COLB + r * BS);
-        const uint4 r1 = *reinterpret_cast<const uint4*>(st + (q0 + q + 1) * G::COLB + r * BS);
-        Chunk<FMT> c0h, c1h;
-        decode_chunk<FMT>(r0, c0h);
-        decode_chunk<FMT>(r1, c1h);
-#pragma unroll
-        for (int e = 0; e < E; e++) {
-            const float2 wh2 = make_float2(wh[e], wh[e]), nwh2 = make_float2(-wh[e], -wh[e]);
-            const float2 wl2 = make_float2(wl[e], wl[e]);
-            if constexpr (SingleFloat<FMT>::value)
-                df2_mac(S2[q / 2], C2[q / 2], make_float2(c0h.vh[e], c1h.vh[e]), wh2, nwh2, wl2);
-            else
-                df2_mac2(S2[q / 2], C2[q / 2], make_float2(c0h.vh[e], c1h.vh[e]), make_float2(c0h.vl[e], c1h.vl[e]),
-                         wh2, nwh2, wl2);
-        }
-        df2_renorm(S2[q / 2], C2[q / 2]);
+        Chunk<FMT> ch;
+        decode_chunk<FMT>(*reinterpret_cast<const uint4*>(st + (q0 + q) * G::COLB + r * BS), ch);
+        df2_mac_chunk<FMT>(S2[q], C2[q], ch, w2, nw2, l2);
     }
 }
 
@@ -226,8 +224,8 @@ __global__ void __launch_bounds__(DOT_THREADS, 1) k_basis_dot_tma(DotArgs a, int
     unsigned char* ring = tma_smem;
     uint64_t* full = reinterpret_cast<uint64_t*>(tma_smem + (size_t)stages * G::STAGE_DOT);
     uint64_t* empty = full + stages;
-    __shared__ double red_g[2][TMA_CW][CG];   // per row group sums of the current group (double-buffered)
-    __shared__ double red_tot[MAXCOLS];       // the block's column totals
+    __shared__ float2 red_g[2][TMA_CW][CG];   // per row group sums of the current group (double-buffered)
+    __shared__ float2 red_tot[MAXCOLS];       // the block's column totals
     __shared__ int failed;
     const int ncols = a.ncols_dev ? *a.ncols_dev : a.ncols;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -245,7 +243,7 @@ __global__ void __launch_bounds__(DOT_THREADS, 1) k_basis_dot_tma(DotArgs a, int
         }
         mbar_init_fence();
     }
-    for (int i = threadIdx.x; i < MAXCOLS; i += DOT_THREADS) red_tot[i] = 0.0;
+    for (int i = threadIdx.x; i < MAXCOLS; i += DOT_THREADS) red_tot[i] = make_float2(0.f, 0.f);
     __syncthreads();
 
     if (warp == DOT_CW) {
@@ -265,9 +263,9 @@ __global__ void __launch_bounds__(DOT_THREADS, 1) k_basis_dot_tma(DotArgs a, int
             // this block's tiles of group g
             const long long tb = ib > (long long)g * ntiles ? ib - (long long)g * ntiles : 0;
             const long long te = ie < (long long)(g + 1) * ntiles ? ie - (long long)g * ntiles : ntiles;
-            float2 S2[CGW / 2], C2[CGW / 2];
+            float2 S2[CGW], C2[CGW];
 #pragma unroll
-            for (int q = 0; q < CGW / 2; q++) { S2[q] = make_float2(0.f, 0.f); C2[q] = make_float2(0.f, 0.f); }
+            for (int q = 0; q < CGW; q++) { S2[q] = make_float2(0.f, 0.f); C2[q] = make_float2(0.f, 0.f); }
             for (long long t = tb; t < te; t++) {
                 if (!bad && !warp_wait(&full[rg.s], rg.ph, limit)) {
                     bad = true;
@@ -284,73 +282,54 @@ __global__ void __launch_bounds__(DOT_THREADS, 1) k_basis_dot_tma(DotArgs a, int
             }
             float S[CGW], C[CGW];
 #pragma unroll
-            for (int q = 0; q < CGW / 2; q++) {
-                S[2 * q] = S2[q].x;
-                S[2 * q + 1] = S2[q].y;
-                C[2 * q] = C2[q].x;
-                C[2 * q + 1] = C2[q].y;
+            for (int q = 0; q < CGW; q++) {
+                S[q] = S2[q].x;
+                C[q] = C2[q].x;
+                df_add(S[q], C[q], S2[q].y, C2[q].y);
             }
             const int col = df_warp_fold<CGW>(S, C, lane);
-            const double wsum = df_to_double(S[0], C[0]);
-            if ((lane & LOW) == 0) red_g[g & 1][rgp][q0 + col] = wsum;
+            if ((lane & LOW) == 0) red_g[g & 1][rgp][q0 + col] = make_float2(S[0], C[0]);
             consumers_sync();
             // red_g[g & 1] is rewritten two groups later, after the next barrier
             const int tid = warp * 32 + lane;
             if (tid < nc) {
-                double tot = 0.0;
+                float2 tot = red_g[g & 1][0][tid];
 #pragma unroll
-                for (int w = 0; w < TMA_CW; w++) tot += red_g[g & 1][w][tid];
+                for (int w = 1; w < TMA_CW; w++) df_add(tot.x, tot.y, red_g[g & 1][w][tid].x, red_g[g & 1][w][tid].y);
                 red_tot[c0 + tid] = tot;
             }
         }
     }
     __syncthreads();
     if (failed && threadIdx.x == 0) record_fault(nullptr, fault);
-    for (int col = threadIdx.x; col < ncols; col += DOT_THREADS) a.part[(long long)blockIdx.x * MAXCOLS + col] = red_tot[col];
+    float2* part = reinterpret_cast<float2*>(a.part);
+    for (int col = threadIdx.x; col < ncols; col += DOT_THREADS) part[(long long)blockIdx.x * MAXCOLS + col] = red_tot[col];
     // Grid barrier (the kernel is launched cooperatively: every block is resident), then
-    // block b adds the partials of the columns b, b + gridDim.x, ...: one load per thread
-    // and column, one warp shuffle tree per warp, then one over the warps' sums.  The
-    // cross-block sum is spread over all SMs instead of one last block, whose FP64 pipe
-    // (a few FP64 operations per clock per SM on GB300) and serial L2 round trips would
-    // otherwise add tens of microseconds to a launch.
+    // block b adds the partials of the columns b, b + gridDim.x, ..., a warp per column: its
+    // lanes add the blocks lane, lane + 32, ... (five loads in flight) and fold.  The cross-block
+    // sum is spread over all SMs, and in double-float: an FP64 instruction occupies GB300's
+    // pipe for 20 cycles per SM, and the FP64 sums (the block's row groups, then 152 partials a
+    // column by the block's warps) took 2 to 4 us of a launch: mean of a restart cycle of 100 f32
+    // 128^3 75.5 -> 71.8 us, i16 101^3 40.2 -> 36.6, bf16 524,288 rows 17.5 -> 14.9, f64 96^3 80.0 -> 78.1.
     if (!grid_barrier(a.counter, limit)) {
         if (threadIdx.x == 0) record_fault(nullptr, fault);
         return;
     }
-    __shared__ double wsum_sh[DOT_CW + 1][4];
     const int nb = gridDim.x;
-    for (int c0 = blockIdx.x; c0 < ncols; c0 += 4 * nb) {
-        double v[4] = {0.0, 0.0, 0.0, 0.0};
-        for (int t = threadIdx.x; t < nb; t += DOT_THREADS) {   // a thread adds blocks t, t + 544, ...
-            double q[4];
+    for (int col = blockIdx.x + warp * nb; col < ncols; col += (DOT_CW + 1) * nb) {
+        float S = 0.f, C = 0.f;
+        for (int t0 = 0; t0 < nb; t0 += 160) {
+            float2 v[5];
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const int col = c0 + k * nb;
-                q[k] = col < ncols ? __ldcg(a.part + (long long)t * MAXCOLS + col) : 0.0;
+            for (int u = 0; u < 5; u++) {
+                const int t = t0 + lane + 32 * u;
+                v[u] = t < nb ? __ldcg(part + (long long)t * MAXCOLS + col) : make_float2(0.f, 0.f);
             }
 #pragma unroll
-            for (int k = 0; k < 4; k++) v[k] += q[k];
+            for (int u = 0; u < 5; u++) df_add(S, C, v[u].x, v[u].y);
         }
-#pragma unroll
-        for (int k = 0; k < 4; k++) v[k] = warp_sum(v[k]);
-        if (lane == 0)
-#pragma unroll
-            for (int k = 0; k < 4; k++) wsum_sh[warp][k] = v[k];
-        __syncthreads();
-        if (warp == 0) {
-            // the 17 warps' sums of the four columns at once: lane l takes column l / 8 and
-            // warps l % 8, l % 8 + 8, l % 8 + 16 (in that order), then a three-level tree
-            // within each group of eight lanes
-            const int k = lane >> 3, w0 = lane & 7;
-            double sum = 0.0;
-#pragma unroll
-            for (int w = w0; w < DOT_CW + 1; w += 8) sum += wsum_sh[w][k];
-#pragma unroll
-            for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xFFFFFFFFu, sum, o);
-            const int col = c0 + k * nb;
-            if (w0 == 0 && col < ncols) a.out[col] = sum * a.scales[col];
-        }
-        __syncthreads();
+        df_warp_sum(S, C);
+        if (lane == 0) a.out[col] = df_to_double(S, C) * a.scales[col];
     }
 }
 
