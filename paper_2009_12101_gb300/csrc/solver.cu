@@ -745,17 +745,24 @@ void set_format(cbg_handle* h, int fmt)
 
 // Whether a restart cycle runs as one launch (cbg_cycle.cuh), and how.  Measured against the
 // stepwise kernels, whole solves at restart 100 (ms, stepwise -> one launch): 5-point 64^2
-// f64 18.6 -> 4.8, 7-point 31^3 f16 13.9 -> 4.6, 64^3 f32 23.6 -> 14.6, 27 per row at
-// 262144 rows f64 2.75 -> 2.64; beyond CYCLE_MAX_ROWS the stepwise basis kernels, which
-// keep more bytes in flight, take the lead (96^3 f64 123 -> 140).
-constexpr long long CYCLE_MAX_ROWS = 300000;
+// f64 18.6 -> 4.8, 7-point 31^3 f16 13.9 -> 4.6, 64^3 f32 23.6 -> 14.6.  Larger matrices, 200
+// steps: 7-point f32 80^3 27.0 -> 21.7, 96^3 36.5 -> 34.4, 112^3 53.5 -> 54.3; f64 64^3 28.6 ->
+// 26.3, 72^3 37.0 -> 36.9, 80^3 43.5 -> 50.1 (the stepwise kernels keep more bytes in flight);
+// 27 per row f32 262,144 rows 3.0 -> 2.2, 393,216 3.6 -> 3.4, 524,288 4.1 -> 4.1, f64 393,216 rows
+// 3.5 -> 3.9 (they also run the SpMV with three times the warps).  Hence the limits: rows for
+// f64 and for the other formats, and fewer rows where a row is long.
+bool cycle_worthwhile(long long n, long long nnz, int fmt)
+{
+    if (fmt == CBG_F64) return n <= 350000;
+    return n <= 850000 && nnz <= 11000000;
+}
 constexpr int CYCLE_MIN_BLOCK_ROWS = 64;   // fewer blocks cost less in the barriers and sums
                                            // than they save in the products (64^2: 32 rows
                                            // 4.85 ms, 64 4.79, 128 5.02)
 void plan_cycle(cbg_handle* h)
 {
     h->cycle_grid = 0;
-    if (!h->cycle_part) return;
+    if (!h->cycle_part || !cycle_worthwhile(h->n, h->nnz, h->fmt)) return;
     const Ops& op = ops_for(h->fmt);
     const int mcols = (int)round_up(h->m + 1, 32);
     const int blocks = std::min(num_sms(), CY_MAXG);
@@ -1485,7 +1492,7 @@ int cbgmres_create(const cbg_csr* A, int restart, int fmt, const cbg_options* op
     // one launch per restart cycle: the default arithmetic and orthogonalisation; profiling
     // times the kernels of a step, so it keeps them apart
     const bool single = o.arith == CBG_ARITH_DF32 && o.ortho == CBG_ORTHO_CGS && o.reorth == CBG_REORTH_ALWAYS &&
-                        h->valdf && !o.profile && n <= CYCLE_MAX_ROWS;
+                        h->valdf && !o.profile && cycle_worthwhile(n, nnz, fmt);
     size_t o_cyc = single ? take(sizeof(float2) * (CY_PART + CY_NORM + CY_COEF)) : 0;
     unsigned char* blk = nullptr;
     TRY(dalloc(&blk, off));

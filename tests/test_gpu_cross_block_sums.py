@@ -1,6 +1,6 @@
 """The sums over blocks of the stepwise kernels in double-float (column sums of the pipelined
 dot, ||w|| of the axpy, omega of the SpMV) against FP64 arithmetic, from two rows to more blocks
-than SMs."""
+than SMs, and the row limits between the stepwise kernels and the single-launch cycle."""
 import numpy as np
 import pytest
 
@@ -30,3 +30,25 @@ def test_block_sums_match_fp64(fmt, n):
             H.append(s.arnoldi(b, x0, k))
     # both evaluate the same columns to FP64 class, the bar the solver is held to everywhere
     assert col_relerr(H[0], H[1], k).max() <= 1e-10
+
+
+@pytest.mark.parametrize("fmt,n,single", [("f64", 350000, True), ("f64", 350001, False), ("f16", 849999, True),
+                                          ("f32", 850000, True), ("f32", 850001, False), ("i16", 600007, True)])
+def test_row_limits_of_the_single_launch(fmt, n, single):
+    """Either side of the limits: the same columns as the stepwise kernels, and the route."""
+    torch, cb = need_gpu()
+    A = _tridiagonal(n)
+    b = to_dev(torch, W.random_vector(n, 3))
+    out = []
+    for profile in (False, True):
+        with cb.Solver.from_csr(A, restart=12, fmt=fmt, profile=profile) as s:
+            x = torch.zeros_like(b)
+            H = s.arnoldi(b, x, 10)
+            st = s.solve(b, x, tol=1e-9, maxit=2000)
+            out.append((H, st, x))
+    (Hc, sc, xc), (Hs, ss, xs) = out
+    assert col_relerr(Hc, Hs, Hc.shape[1]).max() <= 1e-10
+    assert sc["status"] == ss["status"] == 0
+    assert (sc["kernel_launches"] < ss["kernel_launches"]) == single
+    # diagonally dominant by 0.9 of a norm of 5.1: residuals of 1e-9 ||b|| each
+    assert float((xc - xs).norm()) <= 2e-9 / 0.9 * float(b.norm())
