@@ -17,6 +17,9 @@ template <int FMT> struct Launcher {
     // bulk-copy pipelined DF32 dot (one block per SM)
     static void dot_tma(int grid, cudaStream_t s, const DotArgs& a, int* fault);
     static bool tma_fits();
+    // the first pass's subtraction and the second pass's projection in one pass over the basis
+    static void pass(int grid, cudaStream_t s, const PassArgs& a, int* fault);
+    static bool pass_fits(int ncols);
     static void store(int grid, cudaStream_t s, const StoreArgs& a);
     static void spmv_code(int mode, int group, int grid, cudaStream_t s, const SpmvArgs& a);
     // per-step SpMV on the sliced-ELL copy (Arnoldi mode, double-float rows)

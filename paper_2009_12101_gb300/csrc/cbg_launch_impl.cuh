@@ -78,6 +78,48 @@ template <int FMT> void Launcher<FMT>::dot_tma(int grid, cudaStream_t s, const D
     cudaLaunchKernelEx(&cfg, k_basis_dot_tma<FMT>, a, p.stages, fault);
 }
 
+template <int FMT, int RS> static bool pass_kernel_fits()
+{
+    static const bool ok = [] {
+        cudaFuncAttributes fa{};
+        const bool good = cudaFuncGetAttributes(&fa, k_basis_pass<FMT, RS>) == cudaSuccess &&
+                          (int)fa.sharedSizeBytes <= PassGeom<FMT>::STATIC &&
+                          cudaFuncSetAttribute(k_basis_pass<FMT, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               TMA_SMEM_OPTIN - PassGeom<FMT>::STATIC) == cudaSuccess;
+        if (!good) cudaGetLastError();
+        return good;
+    }();
+    return ok;
+}
+
+template <int FMT> bool Launcher<FMT>::pass_fits(int ncols)
+{
+    return PassGeom<FMT>::holds(ncols, 1) && pass_kernel_fits<FMT, 1>() && pass_kernel_fits<FMT, 2>() &&
+           pass_kernel_fits<FMT, 4>() && pass_kernel_fits<FMT, 8>();
+}
+
+template <int FMT> void Launcher<FMT>::pass(int grid, cudaStream_t s, const PassArgs& a, int* fault)
+{
+    using G = PassGeom<FMT>;
+    const int rs = G::spans(a.d.ncols, a.d.nrows, grid), slots = G::slots(a.d.ncols, rs);
+    cudaLaunchConfig_t cfg{};          // cooperative: as the dot
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(PS_THREADS);
+    cfg.dynamicSmemBytes = (size_t)PS_WARPS * slots * 512 + G::fixed(rs);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    switch (rs) {
+    case 1: cudaLaunchKernelEx(&cfg, k_basis_pass<FMT, 1>, a, slots, fault); break;
+    case 2: cudaLaunchKernelEx(&cfg, k_basis_pass<FMT, 2>, a, slots, fault); break;
+    case 4: cudaLaunchKernelEx(&cfg, k_basis_pass<FMT, 4>, a, slots, fault); break;
+    default: cudaLaunchKernelEx(&cfg, k_basis_pass<FMT, 8>, a, slots, fault); break;
+    }
+}
+
 template <int FMT> void Launcher<FMT>::store(int grid, cudaStream_t s, const StoreArgs& a)
 {
     // mode 0: at least two blocks (block 0 runs the Givens update, the others encode)

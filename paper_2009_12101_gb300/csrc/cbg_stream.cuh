@@ -18,6 +18,9 @@
 // bounded (cbg_tma.cuh): a pipeline that stops making progress records FAULT_TIMEOUT and
 // the kernel returns after draining its own copies.
 #pragma once
+#include <algorithm>
+#include <type_traits>
+
 #include "cbg_kernels.cuh"
 #include "cbg_tma.cuh"
 
@@ -206,6 +209,42 @@ __device__ __forceinline__ void consumers_sync()
     asm volatile("bar.sync 1, %0;" ::"r"(DOT_CW * 32) : "memory");
 }
 
+// The blocks' column totals tot (shared memory, written by all threads before) to
+// a.out = scales .* total.  Grid barrier (the kernels are launched cooperatively: every block
+// is resident), then block b adds the partials of the columns b, b + gridDim.x, ..., a warp per
+// column: its lanes add the blocks lane, lane + 32, ... (five loads in flight) and fold.  The
+// cross-block sum is spread over all SMs, and in double-float: an FP64 instruction occupies
+// GB300's pipe for 20 cycles per SM, and the FP64 sums (the block's row groups, then 152
+// partials a column by the block's warps) took 2 to 4 us of a launch: mean of a restart cycle of
+// 100 f32 128^3 75.5 -> 71.8 us, i16 101^3 40.2 -> 36.6, bf16 524,288 rows 17.5 -> 14.9, f64 96^3
+// 80.0 -> 78.1.
+__device__ __forceinline__ void dot_finish(const DotArgs& a, const float2* tot, int ncols, long long limit, int* fault)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    float2* part = reinterpret_cast<float2*>(a.part);
+    for (int col = threadIdx.x; col < ncols; col += blockDim.x) part[(long long)blockIdx.x * MAXCOLS + col] = tot[col];
+    if (!grid_barrier(a.counter, limit)) {
+        if (threadIdx.x == 0) record_fault(nullptr, fault);
+        return;
+    }
+    const int nb = gridDim.x;
+    for (int col = blockIdx.x + warp * nb; col < ncols; col += nw * nb) {
+        float S = 0.f, C = 0.f;
+        for (int t0 = 0; t0 < nb; t0 += 160) {
+            float2 v[5];
+#pragma unroll
+            for (int u = 0; u < 5; u++) {
+                const int t = t0 + lane + 32 * u;
+                v[u] = t < nb ? __ldcg(part + (long long)t * MAXCOLS + col) : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < 5; u++) df_add(S, C, v[u].x, v[u].y);
+        }
+        df_warp_sum(S, C);
+        if (lane == 0) a.out[col] = df_to_double(S, C) * a.scales[col];
+    }
+}
+
 // DF32 arithmetic; a.wdf (w split into FP32 hi and lo planes) is required.  Sixteen
 // consumer warps: warp w takes rows group (w % 8) of every tile and half (w / 8) of every
 // stage's columns.  At the end of every column group the consumer warps meet once (a
@@ -302,35 +341,401 @@ __global__ void __launch_bounds__(DOT_THREADS, 1) k_basis_dot_tma(DotArgs a, int
     }
     __syncthreads();
     if (failed && threadIdx.x == 0) record_fault(nullptr, fault);
-    float2* part = reinterpret_cast<float2*>(a.part);
-    for (int col = threadIdx.x; col < ncols; col += DOT_THREADS) part[(long long)blockIdx.x * MAXCOLS + col] = red_tot[col];
-    // Grid barrier (the kernel is launched cooperatively: every block is resident), then
-    // block b adds the partials of the columns b, b + gridDim.x, ..., a warp per column: its
-    // lanes add the blocks lane, lane + 32, ... (five loads in flight) and fold.  The cross-block
-    // sum is spread over all SMs, and in double-float: an FP64 instruction occupies GB300's
-    // pipe for 20 cycles per SM, and the FP64 sums (the block's row groups, then 152 partials a
-    // column by the block's warps) took 2 to 4 us of a launch: mean of a restart cycle of 100 f32
-    // 128^3 75.5 -> 71.8 us, i16 101^3 40.2 -> 36.6, bf16 524,288 rows 17.5 -> 14.9, f64 96^3 80.0 -> 78.1.
-    if (!grid_barrier(a.counter, limit)) {
-        if (threadIdx.x == 0) record_fault(nullptr, fault);
-        return;
+    dot_finish(a, red_tot, ncols, limit, fault);
+}
+
+// =============================================== w -= V h, u = V^T w in one pass over V
+// The subtraction of the first CGS pass and the projection of the second one: each row of
+// w - V h needs only that row of V, so a tile of rows that holds all columns in shared memory
+// serves both products, and a step reads the basis three times instead of four.
+//
+// What bounds it: the double-float products, 2 x 11 FP32 operations an element and the
+// decoding (twice; FP64 codes are split once and kept as pairs in place); ncu at 96^3, 96
+// columns: f32 89 us, FMA pipe 66 %, f64 160 us, issue 62 %, a tile's barriers 15 to 10 % of the
+// stalls.  Mean over a restart cycle of 100, this pass against the axpy and the dot that it
+// replaces: f32 128^3 150 -> 117 us, 96^3 76 -> 58; f64 276 -> 206, 132 -> 95; f16 131 -> 120,
+// 67 -> 62; i16 137 -> 124; i32 164 -> 148; e4m3 133 -> 128; never slower from 27,000 rows (f32 25 -> 15)
+// to 2,097,152 and from 16 to 112 columns.
+//
+// Sixteen warps in two groups of eight; a group works on its own tile, so one group's
+// products cover the other's barriers.  A tile is `rs` spans of 512 bytes of codes per
+// column (32 lanes x 16 bytes), all columns; warp w of a group takes the span w / sets and
+// the columns w % sets, w % sets + sets, ... (sets = 8 / rs).  Few columns take more spans: the
+// tile stays large and the warps' partial rows few.  rs is a template parameter: with it
+// at run time the divisions and strides took a third of the instructions (f32 128^3 150 us,
+// no gain).  Every thread copies (cp.async) exactly the codes that it reads, into slots of
+// its warp, so the copies need no barrier; bulk copies of 512 bytes a column took 80 cycles
+// each to issue.
+// Phase A: the lane's rows of V h over its columns; the sets' partial rows meet in shared
+// memory, where w is updated, and in memory.  Phase B: the same codes times the new w,
+// accumulated per column in registers over all tiles of the block; a slot read here
+// takes its next column at once.
+constexpr int PS_GROUPS = 2, PS_GW = 8;          // groups, warps of a group
+constexpr int PS_WARPS = PS_GROUPS * PS_GW, PS_THREADS = PS_WARPS * 32;   // 128 registers a thread
+constexpr int PS_NCW = 14;                       // columns of a warp (register accumulators: 56 of 128)
+constexpr int PS_MAXC = PS_GW * PS_NCW;          // columns the pass can hold
+
+// Shared memory: slots [warps][slots][512 B] | per group: partial rows, sets x (rows + pad)
+// floats for S, again for C, then the new w's planes | coefficients.
+template <int FMT> struct PassGeom {
+    static constexpr int BS = FmtInfo<FMT>::bytes;
+    static constexpr int E = 16 / BS;
+    static constexpr int SPAN = 32 * E;                            // rows of a span
+    static constexpr int HE = E > 8 ? 8 : E;                       // rows a lane works on at a time
+    static constexpr int COEF = PS_MAXC * 24;
+    static constexpr int STATIC = PS_WARPS * 16 * 8 + PS_MAXC * 8 + 128;
+    // threads that add one row's sets
+    static constexpr __host__ __device__ int lanes(int rs)
+    {
+        const int sets = PS_GW / rs, t = PS_GW * 32 / (rs * SPAN);
+        return t < 1 ? 1 : (t < sets ? t : sets);
     }
-    const int nb = gridDim.x;
-    for (int col = blockIdx.x + warp * nb; col < ncols; col += (DOT_CW + 1) * nb) {
-        float S = 0.f, C = 0.f;
-        for (int t0 = 0; t0 < nb; t0 += 160) {
-            float2 v[5];
+    static constexpr __host__ __device__ int exld(int rs) { return rs * SPAN + 32 / lanes(rs); }
+    static constexpr __host__ __device__ int exch_floats(int rs)
+    {
+        const int sets = PS_GW / rs;
+        return (sets > 1 ? 2 * sets * exld(rs) : 0) + 2 * rs * SPAN;
+    }
+    static int warp_cols(int ncols, int rs) { return (ncols + PS_GW / rs - 1) / (PS_GW / rs); }
+    static size_t fixed(int rs) { return (size_t)PS_GROUPS * exch_floats(rs) * 4 + COEF; }
+    static int room(int rs) { return (int)((TMA_SMEM_OPTIN - STATIC - fixed(rs)) / (PS_WARPS * 512)); }
+    // slots of a warp: the tile at work and (part of) the next one
+    static int slots(int ncols, int rs) { return std::min(room(rs), 2 * warp_cols(ncols, rs)); }
+    // whether `rs` spans hold all columns, with at least two slots for the next tile
+    static bool holds(int ncols, int rs) { return warp_cols(ncols, rs) <= PS_NCW && warp_cols(ncols, rs) + 2 <= room(rs); }
+    // the widest tile that leaves every block five of them (two groups): 16 of them was slower
+    // (16 columns, 96^3: f16 31 -> 24 us, f32 28 -> 23), and as a rule on columns alone the last
+    // tiles would leave half of the chip idle
+    static int spans(int ncols, long long nrows, int grid)
+    {
+        int rs = 8;
+        while (rs > 1 && (!holds(ncols, rs) || nrows / ((long long)rs * SPAN) < 5LL * grid)) rs >>= 1;
+        return rs;
+    }
+};
+
+struct PassArgs {
+    DotArgs d;                // V, ldb, ncols, scales, nrows, part, active, counter; out = u
+    const double* coef;       // h of the first pass
+    float* wdf;               // w's planes, read and overwritten with w - V h
+};
+
+__device__ __forceinline__ void group_sync(int g)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + g), "r"(PS_GW * 32) : "memory");
+}
+
+__device__ __forceinline__ void async_copy16(unsigned dst, const void* src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// P float pairs to p (8*P-byte aligned) with vector stores
+template <int P> __device__ __forceinline__ void store_pairs(float* p, const float2* v)
+{
+    if constexpr (P == 1) *reinterpret_cast<float2*>(p) = v[0];
+    else {
 #pragma unroll
-            for (int u = 0; u < 5; u++) {
-                const int t = t0 + lane + 32 * u;
-                v[u] = t < nb ? __ldcg(part + (long long)t * MAXCOLS + col) : make_float2(0.f, 0.f);
-            }
+        for (int e = 0; e < P; e += 2)
+            *reinterpret_cast<float4*>(p + 2 * e) = make_float4(v[e].x, v[e].y, v[e + 1].x, v[e + 1].y);
+    }
+}
+
+// HE rows of one column as float pairs (1-byte codes: 8 of a chunk's 16 rows).  SPLIT: FP64
+// codes were replaced by their pairs
+template <int FMT> __device__ __forceinline__ uint4 pass_load(unsigned p)
+{
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if constexpr (PassGeom<FMT>::E > PassGeom<FMT>::HE)
+        asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(p) : "memory");
+    else
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(p) : "memory");
+    return v;
+}
+template <int FMT, bool SPLIT> __device__ __forceinline__ void pass_decode(const uint4& raw, float2* vh, float2* vl)
+{
+    constexpr int E = PassGeom<FMT>::E, HE = PassGeom<FMT>::HE;
+    if constexpr (FMT == F64 && SPLIT) {
+        vh[0] = make_float2(__uint_as_float(raw.x), __uint_as_float(raw.y));
+        vl[0] = make_float2(__uint_as_float(raw.z), __uint_as_float(raw.w));
+    } else if constexpr (E > HE) {
+        const unsigned w[2] = {raw.x, raw.y};
 #pragma unroll
-            for (int u = 0; u < 5; u++) df_add(S, C, v[u].x, v[u].y);
+        for (int k = 0; k < 2; k++) {
+            dec_e4m3x2(w[k] & 0xFFFFu, vh[2 * k].x, vh[2 * k].y);
+            dec_e4m3x2(w[k] >> 16, vh[2 * k + 1].x, vh[2 * k + 1].y);
         }
-        df_warp_sum(S, C);
-        if (lane == 0) a.out[col] = df_to_double(S, C) * a.scales[col];
+    } else {
+        Chunk<FMT> ch;
+        decode_chunk<FMT>(raw, ch);
+#pragma unroll
+        for (int e = 0; e < E; e += 2) {
+            vh[e / 2] = make_float2(ch.vh[e], ch.vh[e + 1]);
+            if constexpr (!SingleFloat<FMT>::value) vl[e / 2] = make_float2(ch.vl[e], ch.vl[e + 1]);
+        }
     }
+}
+
+template <int FMT, int rs>
+__global__ void __launch_bounds__(PS_THREADS, 1) k_basis_pass(PassArgs a, int slots, int* fault)
+{
+    if (a.d.active && *a.d.active == 0) return;
+    using G = PassGeom<FMT>;
+    constexpr int E = G::E, HE = G::HE, SPAN = G::SPAN;
+    constexpr bool SF = SingleFloat<FMT>::value;
+    extern __shared__ __align__(128) unsigned char tma_smem[];
+    constexpr int rows = rs * SPAN, sets = PS_GW / rs, tpr = G::lanes(rs), exld = G::exld(rs);
+    const int ncols = a.d.ncols;
+    // (the shuffle tells the compiler that everything derived from the warp index is uniform)
+    const int lane = threadIdx.x & 31, warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int g = warp / PS_GW, gw = warp % PS_GW, set = gw % sets, span = gw / sets;
+    const int nq = ncols > set ? (ncols - set + sets - 1) / sets : 0;     // this warp's columns
+    const int gt = threadIdx.x & (PS_GW * 32 - 1);                        // thread of the group
+    const int r0 = (span * 32 + lane) * E;                                // first row of this lane in the tile
+    float* exS = reinterpret_cast<float*>(tma_smem + (size_t)PS_WARPS * slots * 512) + g * G::exch_floats(rs);
+    float* exC = exS + sets * exld;
+    float* wt = exS + (sets > 1 ? 2 * sets * exld : 0);                   // the new w's planes
+    float4* ca = reinterpret_cast<float4*>(tma_smem + (size_t)PS_WARPS * slots * 512 +
+                                           PS_GROUPS * G::exch_floats(rs) * 4);      // (c, c, -c, -c)
+    float2* cb = reinterpret_cast<float2*>(ca + PS_MAXC);                            // (c low, c low)
+    __shared__ float2 red_w[PS_WARPS][16];
+    __shared__ float2 red_tot[PS_MAXC];
+    const long long limit = a.d.wait_limit > 0 ? a.d.wait_limit : WAIT_LIMIT_CYCLES;
+    long long tb, te;
+    block_items(a.d.nrows / rows, tb, te);
+
+    // The warp's slots.  Column q of a tile lies in slot q; the first `ahead` columns (a multiple
+    // of four, or all) alternate with the slots nq + q from tile to tile, so that they can be
+    // copied a tile earlier.  A slot read for the last time takes its next column at once.
+    const unsigned slot0 = smem_addr(tma_smem) + (unsigned)(warp * slots * 512 + lane * 16);
+    int ahead = slots - nq;
+    ahead = ahead >= nq ? nq : ahead & ~3;
+    const long long cstep = (long long)sets * a.d.ldb, tstep = (long long)PS_GROUPS * rs * 512;
+    const unsigned char* src = a.d.V + set * a.d.ldb + (span * 32 + lane) * 16 + (tb + g) * (rs * 512);
+    // copies are committed as: a tile's first columns, its others, the next tile's first columns
+    if (tb + g < te)
+        for (int i = 0; i < ahead; i++) async_copy16(slot0 + i * 512, src + i * cstep);
+    async_commit();
+    if (tb + g < te)
+        for (int i = ahead; i < nq; i++) async_copy16(slot0 + i * 512, src + i * cstep);
+    async_commit();
+    if (tb + g + PS_GROUPS < te)
+        for (int i = 0; i < ahead; i++) async_copy16(slot0 + (nq + i) * 512, src + tstep + i * cstep);
+    async_commit();
+    // coefficients in the order of use: [set][q]
+    for (int k = threadIdx.x; k < PS_MAXC; k += PS_THREADS) {
+        float h = 0.f, l = 0.f;
+        if (k < ncols) split_f64(-a.d.scales[k] * a.coef[k], h, l);
+        const int at = (k % sets) * PS_NCW * rs + k / sets;
+        ca[at] = make_float4(h, h, -h, -h);
+        cb[at] = make_float2(l, l);
+    }
+    __syncthreads();
+
+    float2 S2[PS_NCW], C2[PS_NCW];
+#pragma unroll
+    for (int q = 0; q < PS_NCW; q++) { S2[q] = make_float2(0.f, 0.f); C2[q] = make_float2(0.f, 0.f); }
+    const float4* const wca = ca + set * PS_NCW * rs;
+    const float2* const wcb = cb + set * PS_NCW * rs;
+    unsigned first = slot0;                       // slots of the first columns: slot0 or slot0 + nq * 512
+    float* wg = a.wdf + (tb + g) * rows;
+    for (int left = (int)((te - tb - g + PS_GROUPS - 1) / PS_GROUPS); left > 0; left--, wg += PS_GROUPS * rows) {
+        // the row that this thread will update, ahead of its use
+        float w0h = 0.f, w0l = 0.f;
+        if (sets > 1 && gt % tpr == 0) {
+            w0h = __ldcg(wg + gt / tpr);
+            w0l = __ldcg(wg + a.d.nrows + gt / tpr);
+        }
+        // ---- phase A: rows of V c over this warp's columns
+        async_wait<2>();
+#pragma unroll
+        for (int hf = 0; hf < E / HE; hf++) {
+            constexpr int P = HE / 2, NA = P == 1 ? 2 : 1;   // FP64: two chains of sums
+            float2 A2[NA * P], B2[NA * P];
+#pragma unroll
+            for (int e = 0; e < NA * P; e++) { A2[e] = make_float2(0.f, 0.f); B2[e] = make_float2(0.f, 0.f); }
+            auto columns = [&](int q0, auto count) {              // the codes of a few columns, then their products
+                constexpr int N = decltype(count)::value;
+                const unsigned p = (q0 < ahead ? first : slot0) + (unsigned)q0 * 512u;
+                uint4 raw[N];
+                float4 c4[N];
+                float2 cl[N];
+#pragma unroll
+                for (int u = 0; u < N; u++) {
+                    raw[u] = pass_load<FMT>(p + u * 512 + hf * 8);
+                    c4[u] = wca[q0 + u];
+                    cl[u] = wcb[q0 + u];
+                }
+                float2 vh[N][P], vl[N][SF ? 1 : P];
+#pragma unroll
+                for (int u = 0; u < N; u++) {
+                    pass_decode<FMT, false>(raw[u], vh[u], vl[u]);
+                    const float2 ch = make_float2(c4[u].x, c4[u].y), nch = make_float2(c4[u].z, c4[u].w);
+#pragma unroll
+                    for (int e = 0; e < P; e++) {
+                        const int x = (u % NA) * P + e;
+                        if constexpr (SF) df2_mac(A2[x], B2[x], vh[u][e], ch, nch, cl[u]);
+                        else df2_mac2(A2[x], B2[x], vh[u][e], vl[u][e], ch, nch, cl[u]);
+                    }
+                }
+                if constexpr (FMT == F64) {
+#pragma unroll
+                    for (int u = 0; u < N; u++)
+                        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(p + u * 512), "f"(vh[u][0].x),
+                                     "f"(vh[u][0].y), "f"(vl[u][0].x), "f"(vl[u][0].y)
+                                     : "memory");
+                }
+            };
+            auto renorm = [&] {
+#pragma unroll
+                for (int e = 0; e < NA * P; e++) df2_renorm(A2[e], B2[e]);
+            };
+            int q = 0;
+            for (; q + 4 <= nq; q += 4) {
+                if (q + 4 > ahead) async_wait<1>();
+                if constexpr (SF) {
+                    columns(q, std::integral_constant<int, 4>{});
+                } else {                     // (pairs of floats: registers for two columns at a time)
+                    columns(q, std::integral_constant<int, 2>{});
+                    columns(q + 2, std::integral_constant<int, 2>{});
+                }
+                renorm();
+            }
+            async_wait<1>();
+            for (; q < nq; q++) columns(q, std::integral_constant<int, 1>{});
+            renorm();
+            if constexpr (NA == 2) {
+                df_add(A2[0].x, B2[0].x, A2[1].x, B2[1].x);
+                df_add(A2[0].y, B2[0].y, A2[1].y, B2[1].y);
+            }
+            const int r = r0 + hf * HE;
+            if (sets > 1) {
+                store_pairs<HE / 2>(exS + set * exld + r, A2);
+                store_pairs<HE / 2>(exC + set * exld + r, B2);
+            } else {                    // all columns are this lane's own
+#pragma unroll
+                for (int e = 0; e < HE / 2; e++) {
+                    const float2 wh = *reinterpret_cast<const float2*>(wg + r + 2 * e);
+                    const float2 wl = *reinterpret_cast<const float2*>(wg + a.d.nrows + r + 2 * e);
+                    df_add(A2[e].x, B2[e].x, wh.x, wl.x);
+                    df_add(A2[e].y, B2[e].y, wh.y, wl.y);
+                    df2_renorm(A2[e], B2[e]);
+                }
+                store_pairs<HE / 2>(wt + r, A2);
+                store_pairs<HE / 2>(wt + rows + r, B2);
+                store_pairs<HE / 2>(wg + r, A2);
+                store_pairs<HE / 2>(wg + a.d.nrows + r, B2);
+            }
+        }
+        if (sets > 1) {
+            group_sync(g);
+            const int part = gt % tpr;
+#pragma unroll
+            for (int i = 0; i < rows / (PS_GW * 32 / tpr); i++) {
+                const int r = gt / tpr + i * (PS_GW * 32 / tpr);
+                const float* e = exS + part * exld + r;
+                float s = e[0], c = e[sets * exld];
+#pragma unroll
+                for (int k = tpr; k < sets; k += tpr) df_add(s, c, e[k * exld], e[(sets + k) * exld]);
+#pragma unroll
+                for (int o = 1; o < tpr; o <<= 1) {
+                    const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
+                    df_add(s, c, s2, c2);
+                }
+                if (part == 0) {
+                    if (i > 0) {
+                        w0h = __ldcg(wg + r);
+                        w0l = __ldcg(wg + a.d.nrows + r);
+                    }
+                    df_add(s, c, w0h, w0l);
+                    float h, l;
+                    two_sum(s, c, h, l);
+                    wt[r] = h;
+                    wt[rows + r] = l;
+                    wg[r] = h;
+                    wg[a.d.nrows + r] = l;
+                }
+            }
+            group_sync(g);
+        }
+        // ---- phase B: the warp's columns times the new w, last column first; their slots take
+        // the next tile's columns, those of the first columns the tile's after that
+        const bool more1 = left > 1, more2 = left > 2;
+        if (ahead >= nq) async_commit();
+#pragma unroll
+        for (int hf = 0; hf < E / HE; hf++) {
+            constexpr int U = HE > 4 ? 2 : 4;
+            const int r = r0 + hf * HE;
+            float2 w2[HE / 2], nw2[HE / 2], l2[HE / 2];
+            load_floats<HE>(wt + r, reinterpret_cast<float*>(w2));
+            load_floats<HE>(wt + rows + r, reinterpret_cast<float*>(l2));
+#pragma unroll
+            for (int e = 0; e < HE / 2; e++) nw2[e] = make_float2(-w2[e].x, -w2[e].y);
+#pragma unroll
+            for (int q0 = (PS_NCW - 1) / U * U; q0 >= 0; q0 -= U) {
+                if (q0 < nq) {
+                    const bool fst = q0 < ahead, more = fst ? more2 : more1;
+                    const unsigned p = (fst ? first : slot0) + (unsigned)q0 * 512u;
+                    const unsigned char* np = src + (fst ? 2 * tstep : tstep) + q0 * cstep;
+                    auto group = [&](auto whole) {
+                        constexpr bool W = decltype(whole)::value;       // all U columns exist
+                        uint4 raw[U];
+#pragma unroll
+                        for (int u = 0; u < U; u++)
+                            if (q0 + u < PS_NCW && (W || q0 + u < nq)) raw[u] = pass_load<FMT>(p + u * 512 + hf * 8);
+#pragma unroll
+                        for (int u = 0; u < U; u++) {
+                            if (q0 + u < PS_NCW && (W || q0 + u < nq)) {
+                                const int q = q0 + u;
+                                float2 vh[HE / 2], vl[SF ? 1 : HE / 2];
+                                pass_decode<FMT, true>(raw[u], vh, vl);
+#pragma unroll
+                                for (int e = 0; e < HE / 2; e++) {
+                                    if constexpr (SF) df2_mac(S2[q], C2[q], vh[e], w2[e], nw2[e], l2[e]);
+                                    else df2_mac2(S2[q], C2[q], vh[e], vl[e], w2[e], nw2[e], l2[e]);
+                                }
+                                df2_renorm(S2[q], C2[q]);
+                                if (!W && hf == E / HE - 1 && more) async_copy16(p + u * 512, np + u * cstep);
+                            }
+                        }
+                        if (W && hf == E / HE - 1 && more) {
+#pragma unroll
+                            for (int u = 0; u < U; u++)
+                                if (q0 + u < PS_NCW) async_copy16(p + u * 512, np + u * cstep);
+                        }
+                    };
+                    if (q0 + U <= nq) group(std::true_type{});
+                    else group(std::false_type{});
+                    if (hf == E / HE - 1 && q0 == ahead) async_commit();
+                }
+            }
+        }
+        async_commit();
+        src += tstep;
+        first = first == slot0 ? slot0 + (unsigned)nq * 512u : slot0;
+    }
+    async_wait<0>();
+    float S[16], C[16];
+#pragma unroll
+    for (int q = 0; q < 16; q++) {
+        S[q] = q < PS_NCW ? S2[q < PS_NCW ? q : 0].x : 0.f;
+        C[q] = q < PS_NCW ? C2[q < PS_NCW ? q : 0].x : 0.f;
+        if (q < PS_NCW) df_add(S[q], C[q], S2[q].y, C2[q].y);
+    }
+    const int q = df_warp_fold<16>(S, C, lane);
+    if ((lane & fold_low<16>()) == 0) red_w[warp][q] = make_float2(S[0], C[0]);
+    __syncthreads();
+    for (int c = threadIdx.x; c < ncols; c += PS_THREADS) {
+        float2 tot = make_float2(0.f, 0.f);
+        for (int w = c % sets; w < PS_WARPS; w += sets) df_add(tot.x, tot.y, red_w[w][c / sets].x, red_w[w][c / sets].y);
+        red_tot[c] = tot;
+    }
+    __syncthreads();
+    dot_finish(a.d, red_tot, ncols, limit, fault);
 }
 
 }  // namespace cbg

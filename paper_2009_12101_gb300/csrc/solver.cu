@@ -79,6 +79,8 @@ struct Ops {
     void (*axpy)(int, int, int, cudaStream_t, const AxpyArgs&);
     void (*dot_tma)(int, cudaStream_t, const DotArgs&, int*);
     bool (*tma_fits)();
+    void (*pass)(int, cudaStream_t, const PassArgs&, int*);
+    bool (*pass_fits)(int);
     void (*store)(int, cudaStream_t, const StoreArgs&);
     void (*spmv_code)(int, int, int, cudaStream_t, const SpmvArgs&);
     void (*spmv_sell)(int, cudaStream_t, const SellArgs&);
@@ -95,7 +97,7 @@ struct Ops {
 template <int F> Ops make_ops()
 {
     return Ops{&Launcher<F>::dot, &Launcher<F>::axpy, &Launcher<F>::dot_tma,
-               &Launcher<F>::tma_fits, &Launcher<F>::store, &Launcher<F>::spmv_code, &Launcher<F>::spmv_sell,
+               &Launcher<F>::tma_fits, &Launcher<F>::pass, &Launcher<F>::pass_fits, &Launcher<F>::store, &Launcher<F>::spmv_code, &Launcher<F>::spmv_sell,
                &Launcher<F>::encode, &Launcher<F>::decode, &Launcher<F>::occupancy_dot,
                &Launcher<F>::occupancy_axpy, &Launcher<F>::occupancy_spmv, &Launcher<F>::cycle,
                &Launcher<F>::cycle_fits, &CycleGeom<F>::smem};
@@ -744,17 +746,20 @@ void set_format(cbg_handle* h, int fmt)
 }
 
 // Whether a restart cycle runs as one launch (cbg_cycle.cuh), and how.  Measured against the
-// stepwise kernels, whole solves at restart 100 (ms, stepwise -> one launch): 5-point 64^2
-// f64 18.6 -> 4.8, 7-point 31^3 f16 13.9 -> 4.6, 64^3 f32 23.6 -> 14.6.  Larger matrices, 200
-// steps: 7-point f32 80^3 27.0 -> 21.7, 96^3 36.5 -> 34.4, 112^3 53.5 -> 54.3; f64 64^3 28.6 ->
-// 26.3, 72^3 37.0 -> 36.9, 80^3 43.5 -> 50.1 (the stepwise kernels keep more bytes in flight);
-// 27 per row f32 262,144 rows 3.0 -> 2.2, 393,216 3.6 -> 3.4, 524,288 4.1 -> 4.1, f64 393,216 rows
-// 3.5 -> 3.9 (they also run the SpMV with three times the warps).  Hence the limits: rows for
-// f64 and for the other formats, and fewer rows where a row is long.
-bool cycle_worthwhile(long long n, long long nnz, int fmt)
+// stepwise kernels, 200 steps at restart 100 (ms, stepwise -> one launch), 7-point matrices:
+// f64 48^3 15.2 -> 11.9, 56^3 19.2 -> 20.1, 64^3 23.3 -> 25.3; f32 64^3 15.9 -> 11.8, 80^3 23.6 ->
+// 21.7, 88^3 28.2 -> 29.5; i32 80^3 27.2 -> 25.1, 88^3 32.6 -> 33.9; f16 80^3 22.2 -> 19.4, 88^3 27.4 ->
+// 26.3; i16 88^3 28.6 -> 28.9; restart 25: f64 80^3 4.8 -> 4.6, f32 80^3 3.8 -> 2.5.  27 per row,
+// restart 30: f64 131,072 rows 4.5 -> 3.7, 262,144 6.4 -> 7.2; f32 262,144 5.6 -> 4.5, 393,216 6.5 -> 6.7; bf16
+// 5.5 -> 4.7, 6.7 -> 7.2.  The single launch reads the basis four times a step out of L2, the
+// stepwise kernels three times with more bytes in flight and more warps in the SpMV: hence
+// limits on the basis's bytes (about the L2 for f64; the 4-byte formats' shares on chip reach
+// further), the rows and the nonzeros.
+bool cycle_worthwhile(long long n, long long nnz, int m, int fmt)
 {
-    if (fmt == CBG_F64) return n <= 350000;
-    return n <= 850000 && nnz <= 11000000;
+    const double basis = (double)n * (double)(m + 1) * (double)fmt_bytes(fmt);
+    if (fmt == CBG_F64) return n <= 600000 && nnz <= 5000000 && basis <= 120e6;
+    return n <= 600000 && nnz <= 9000000 && basis <= 235e6;
 }
 constexpr int CYCLE_MIN_BLOCK_ROWS = 64;   // fewer blocks cost less in the barriers and sums
                                            // than they save in the products (64^2: 32 rows
@@ -762,7 +767,7 @@ constexpr int CYCLE_MIN_BLOCK_ROWS = 64;   // fewer blocks cost less in the barr
 void plan_cycle(cbg_handle* h)
 {
     h->cycle_grid = 0;
-    if (!h->cycle_part || !cycle_worthwhile(h->n, h->nnz, h->fmt)) return;
+    if (!h->cycle_part || !cycle_worthwhile(h->n, h->nnz, h->m, h->fmt)) return;
     const Ops& op = ops_for(h->fmt);
     const int mcols = (int)round_up(h->m + 1, 32);
     const int blocks = std::min(num_sms(), CY_MAXG);
@@ -1017,7 +1022,10 @@ void enqueue_step(cbg_handle* h, int j)
             xa.reorth_flag = &h->d.st->reorth_now;
             xa.eta = h->opt.eta;
         }
-        launch(h, 1, pass_bytes, [&] { run_axpy(xa); });
+        // DF32, second pass always: this subtraction and the second projection in one pass over
+        // the basis, as long as a tile of all columns fits (112 columns)
+        const bool fused = planes_only && h->use_tma && op.pass_fits(ncols);
+        if (!fused) launch(h, 1, pass_bytes, [&] { run_axpy(xa); });
         if (reorth) {
             // re-orthogonalisation: u = V^T w1 ; w2 = w1 - V u ; (h += u in the store kernel);
             // conditional mode: both kernels skip themselves unless the flag is set
@@ -1026,7 +1034,15 @@ void enqueue_step(cbg_handle* h, int j)
             da.counter = h->d.counters + 3;
             da.out = h->d.u;
             da.active = gate;
-            launch(h, 0, pass_bytes, run_dot);
+            if (fused) {
+                PassArgs pa{};
+                pa.d = da;
+                pa.coef = h->d.h;
+                pa.wdf = wdf;
+                launch(h, 1, pass_bytes, [&] { op.pass(h->grid_tma, s, pa, &h->d.st->fault); });
+            } else {
+                launch(h, 0, pass_bytes, run_dot);
+            }
             xa.coef = h->d.u;
             xa.w_in = planes_only ? nullptr : h->w1;
             xa.wdf_in = planes_only ? wdf : nullptr;
@@ -1492,7 +1508,7 @@ int cbgmres_create(const cbg_csr* A, int restart, int fmt, const cbg_options* op
     // one launch per restart cycle: the default arithmetic and orthogonalisation; profiling
     // times the kernels of a step, so it keeps them apart
     const bool single = o.arith == CBG_ARITH_DF32 && o.ortho == CBG_ORTHO_CGS && o.reorth == CBG_REORTH_ALWAYS &&
-                        h->valdf && !o.profile && cycle_worthwhile(n, nnz, fmt);
+                        h->valdf && !o.profile && cycle_worthwhile(n, nnz, restart, fmt);
     size_t o_cyc = single ? take(sizeof(float2) * (CY_PART + CY_NORM + CY_COEF)) : 0;
     unsigned char* blk = nullptr;
     TRY(dalloc(&blk, off));

@@ -32,16 +32,18 @@ def test_block_sums_match_fp64(fmt, n):
     assert col_relerr(H[0], H[1], k).max() <= 1e-10
 
 
-@pytest.mark.parametrize("fmt,n,single", [("f64", 350000, True), ("f64", 350001, False), ("f16", 849999, True),
-                                          ("f32", 850000, True), ("f32", 850001, False), ("i16", 600007, True)])
-def test_row_limits_of_the_single_launch(fmt, n, single):
+@pytest.mark.parametrize("fmt,n,restart,single", [
+    ("f64", 600000, 12, True), ("f64", 600001, 12, False), ("f16", 599999, 12, True), ("f32", 600000, 12, True),
+    ("f32", 600001, 12, False), ("i16", 600007, 12, False), ("f64", 149999, 99, True), ("f64", 150001, 99, False),
+    ("f32", 587500, 99, True), ("i32", 587501, 99, False)])
+def test_row_limits_of_the_single_launch(fmt, n, restart, single):
     """Either side of the limits: the same columns as the stepwise kernels, and the route."""
     torch, cb = need_gpu()
     A = _tridiagonal(n)
     b = to_dev(torch, W.random_vector(n, 3))
     out = []
     for profile in (False, True):
-        with cb.Solver.from_csr(A, restart=12, fmt=fmt, profile=profile) as s:
+        with cb.Solver.from_csr(A, restart=restart, fmt=fmt, profile=profile) as s:
             x = torch.zeros_like(b)
             H = s.arnoldi(b, x, 10)
             st = s.solve(b, x, tol=1e-9, maxit=2000)
