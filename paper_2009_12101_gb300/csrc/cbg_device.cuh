@@ -441,11 +441,15 @@ template <int FMT> __device__ __forceinline__ void encode_store(void* base, int6
     } else if constexpr (FMT == F16) {
         reinterpret_cast<__half*>(base)[i] = __double2half(v);
     } else if constexpr (FMT == I32 || FMT == I16) {
-        const int mx = FMT == I32 ? 2147483647 : 32767;
-        double t = __dmul_rn(v, p.inv);
-        double mxd = (double)mx;
-        t = t > mxd ? mxd : (t < -mxd ? -mxd : t);
+        // clamp to +-mx on the converted integer (the conversion saturates; a comparison of
+        // doubles is an FP64-pipe operation), a NaN as the conversion leaves it
+        const double t = __dmul_rn(v, p.inv);
+        const bool nan = ((unsigned int)__double2hiint(t) & 0x7FFFFFFFu) + (__double2loint(t) != 0) > 0x7FF00000u;
         int q = __double2int_rn(t);
+        if (!nan) {
+            constexpr int mx = FMT == I32 ? 2147483647 : 32767;
+            q = q > mx ? mx : (q < -mx ? -mx : q);
+        }
         if constexpr (FMT == I32) reinterpret_cast<int*>(base)[i] = q;
         else reinterpret_cast<short*>(base)[i] = (short)q;
     } else if constexpr (FMT == BF16) {
