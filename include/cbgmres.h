@@ -184,7 +184,8 @@ typedef struct {
 
 /* Per-kernel-class timing gathered while options.profile == 1 (accumulated over
  * solves until cbgmres_profile(..., reset = 1)).  Classes: 0 basis dot (V^T w),
- * 1 basis axpy (w - V h), 2 SpMV (Arnoldi and residual), 3 store/finalize, 4 other.
+ * 1 basis axpy (w - V h, and the pass that forms w - V h and V^T of it together),
+ * 2 SpMV (Arnoldi and residual), 3 store/finalize, 4 other.
  * ms: summed CUDA-event durations; bytes: algorithmic HBM bytes (basis codes read for
  * classes 0-1: columns * n * bytes(fmt); CSR + vectors for class 2; codes written plus
  * w read for class 3); launches: count. */

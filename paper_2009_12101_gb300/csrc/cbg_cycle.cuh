@@ -2,7 +2,7 @@
 // launch, for matrices whose steps are bound by launch and synchronisation latency rather
 // than by HBM.
 //
-// The stepwise path issues six dependent kernels per Arnoldi step; each costs 7-17 us on
+// The stepwise path issues five dependent kernels per Arnoldi step; each costs 7-17 us on
 // GB300 however few rows there are (launch, ramp, one grid-wide sum, drain).  Here the
 // blocks stay resident for the whole cycle: block b owns the rows [b R, (b + 1) R) and keeps
 // them of w in shared memory as double-float planes.  A step is four phases, each ended by
@@ -25,7 +25,7 @@
 // splits and epilogues; only the order of the sums differs (block partials are combined as
 // double-float pairs).
 //
-// What bounds it: 64^2 f64, restart 100, takes 18 us per step against 72 us stepwise: 11.5k
+// What bounds it: 64^2 f64, restart 100, takes 18 us per step (72 us as separate kernels): 11.5k
 // of 36k cycles in the four barriers (about 1.4 us each: one release, one poll), 6k in the
 // two sums over the blocks (an L2 round trip and a warp tree each), 11k in the basis
 // products, 3.6k in the SpMV's chain of three loads, 3k in the FP64 root and division of

@@ -10,6 +10,13 @@
     python -m paper_2009_12101_gb300.profile_cases mlp [grid]
         two fused training passes of the per-row network of the learned preconditioner
         on the lognormal cell-centred diffusion grid^3 (default 64)
+    python -m paper_2009_12101_gb300.profile_cases step [format] [grid] [steps]
+        one restart cycle of `steps` (default 100) Arnoldi steps on the convection-diffusion
+        grid^3 (default f32, 96) with the stepwise kernels
+    python -m paper_2009_12101_gb300.profile_cases cycle [format] [grid]
+        one restart cycle of 100 steps in the single launch (default f32, 64)
+    python -m paper_2009_12101_gb300.profile_cases multi [format] [k]
+        the multi-vector product on the CUDA cores, 2^20 x 100 basis (default f32, k = 5)
 
 Every case runs the library's own kernels through the C ABI on cuda:0 and prints "ok".
 """
@@ -86,6 +93,33 @@ def case_mlp(grid: int = 64) -> None:
     sp.close()
 
 
+def case_step(fmt: str = "f32", grid: int = 96, steps: int = 100, stepwise: bool = True) -> None:
+    import torch
+
+    import paper_2009_12101_gb300 as cb
+    import workloads as W
+    A = W.convdiff3d(grid)
+    b = torch.from_numpy(W.rhs_from_solution(A, W.exact_solution(A.n, 2))).cuda()
+    with cb.Solver.from_csr(A, restart=100, fmt=fmt, profile=stepwise) as s:   # (profiling keeps the kernels apart)
+        x = torch.zeros(A.n, dtype=torch.float64, device="cuda")
+        s.solve(b, x, tol=1e-30, maxit=steps)
+
+
+def case_multi(fmt: str = "f32", k: int = 5) -> None:
+    import torch
+
+    import paper_2009_12101_gb300 as cb
+    n, ncols = 1 << 20, 100
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+    v = torch.randn(ncols, n, device="cuda", generator=g) / n ** 0.5
+    V = v.to({"f64": torch.float64, "f32": torch.float32, "f16": torch.float16}[fmt]).contiguous()
+    W = torch.randn(k, n, dtype=torch.float64, device="cuda", generator=g)
+    for _ in range(3):
+        cb.basis_dot_multi(fmt, n, V, n, np.ones(ncols), W, path="cuda")
+    torch.cuda.synchronize()
+
+
 def main(argv) -> int:
     import paper_2009_12101_gb300 as cb
     cb.ensure_built()
@@ -98,6 +132,12 @@ def main(argv) -> int:
         case_spmv(int(argv[1]) if len(argv) > 1 else -1, int(argv[2]) if len(argv) > 2 else 96)
     elif which == "mlp":
         case_mlp(int(argv[1]) if len(argv) > 1 else 64)
+    elif which in ("step", "cycle"):
+        stepwise = which == "step"
+        case_step(argv[1] if len(argv) > 1 else "f32", int(argv[2]) if len(argv) > 2 else (96 if stepwise else 64),
+                  int(argv[3]) if len(argv) > 3 else 100, stepwise)
+    elif which == "multi":
+        case_multi(argv[1] if len(argv) > 1 else "f32", int(argv[2]) if len(argv) > 2 else 5)
     else:
         raise SystemExit(f"unknown case {which}")
     print("ok")
