@@ -404,12 +404,40 @@ struct EncParams {
 // 2^e as an FP64 value built from its bits, for |e| <= 1022
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(1023 + e) << 52); }
 
+// the bits of a double, and 2^e for -1022 <= e <= 1023, on host and device
+__host__ __device__ inline unsigned long long f64_bits(double x)
+{
+    unsigned long long u;
+    memcpy(&u, &x, 8);
+    return u;
+}
+__host__ __device__ inline double pow2_any(int e)
+{
+    if (e < -1022 || e > 1023) return ldexp(1.0, e);
+    const unsigned long long u = (unsigned long long)(1023 + e) << 52;
+    double x;
+    memcpy(&x, &u, 8);
+    return x;
+}
+
+// Smallest integer e with vmax <= fmax * 2^e, at least -126: from the exponents and one
+// comparison of the significands, all on integers (the search by ldexp took some 150
+// operations of the narrow FP64 pipe in every storing block: bf16 27 per row 10.68 -> 10.55 ms,
+// a bf16 solve in the single launch 21.3 -> 19.3); the search remains for subnormal and
+// infinite vmax.
 __host__ __device__ inline int pow2_exponent_for(double vmax, double fmax)
-{   // smallest integer e with vmax <= fmax * 2^e, at least -126
-    int e2;
-    (void)frexp(vmax, &e2);
-    int e = e2 - 12;
-    while (vmax > ldexp(fmax, e)) e += 1;
+{
+    const unsigned long long v = f64_bits(vmax), f = f64_bits(fmax), frac = 0xFFFFFFFFFFFFFull;
+    const int ve = (int)(v >> 52) & 0x7FF, fe = (int)(f >> 52) & 0x7FF;
+    int e;
+    if (ve >= 1 && ve <= 2046) {
+        e = ve - fe + ((v & frac) > (f & frac) ? 1 : 0);
+    } else {
+        int e2;
+        (void)frexp(vmax, &e2);
+        e = e2 - 12;
+        while (vmax > ldexp(fmax, e)) e += 1;
+    }
     if (e < -126) e = -126;
     return e;
 }
@@ -424,8 +452,8 @@ __host__ __device__ inline EncParams enc_params(int fmt, double vmax)
         p.inv = 1.0 / p.scale;
     } else if (fmt == BF16 || fmt == E4M3) {
         int e = pow2_exponent_for(vmax, fmt == BF16 ? 1.0 : 448.0);
-        p.scale = ldexp(1.0, e);
-        p.inv = ldexp(1.0, -e);
+        p.scale = pow2_any(e);
+        p.inv = pow2_any(-e);
     }
     return p;
 }
