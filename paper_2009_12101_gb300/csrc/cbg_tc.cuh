@@ -37,21 +37,6 @@ __host__ __device__ constexpr uint32_t tc_idesc(int M, int N, bool bf16)
     return (1u << 4) | (bf16 ? (1u << 7) | (1u << 10) : 0u) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// The same tile read as an MN-major operand (its 128-byte lines hold 64 values along M or N, a
-// line per K value): lines of K in groups of eight TC_SBO bytes apart, the next 64 values
-// along M or N `next` bytes behind.  One MMA consumes K = 16 lines.  Goes with TC_A_MN /
-// TC_B_MN in the instruction descriptor.
-constexpr uint32_t TC_A_MN = 1u << 15, TC_B_MN = 1u << 16;
-__device__ __forceinline__ uint64_t tc_desc_mn(uint32_t addr, uint32_t next)
-{
-    uint64_t d = (uint64_t)((addr >> 4) & 0x3FFF);
-    d |= (uint64_t)((next >> 4) & 0x3FFF) << 16;
-    d |= (uint64_t)((TC_SBO >> 4) & 0x3FFF) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-
 // D (tensor memory) = A B^T (+ D when acc != 0), issued by one thread
 __device__ __forceinline__ void tc_mma(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, int acc)
 {

@@ -33,8 +33,8 @@ namespace {
 constexpr int LT = 256;            // threads of the row kernels
 
 __global__ void k_spai_setup(const int* rowptr, const int* col, const double* val, long long n, long long sx,
-                             long long sxy, signed char* slot, float* feat, double* diag, float* idiag,
-                             unsigned char* mask, int* bad)
+                             long long sxy, signed char* slot, float* feat, double* diag, unsigned char* mask,
+                             int* bad)
 {
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         const long long off[7] = {-sxy, -sx, -1, 0, 1, sx, sxy};
@@ -53,7 +53,6 @@ __global__ void k_spai_setup(const int* rowptr, const int* col, const double* va
         const double d = a[3];
         if (!(d != 0.0) || !isfinite(d)) atomicExch(bad, 1);
         diag[i] = d;
-        idiag[i] = __frcp_rn(f64_to_f32_rn(d));      // the loss takes 1 / a_ii in FP32
         mask[i] = m;
         for (int k = 0; k < 7; k++) feat[i * 7 + k] = (float)(a[k] / d);
     }
@@ -88,8 +87,8 @@ __global__ void k_pair_residual(const int* rowptr, const int* col, const double*
 
 // add one pair (weight 1/||e||^2, from the block partials) to G, c, d
 __global__ void k_pair_accumulate(const int* rowptr, const int* col, const signed char* slot, long long n,
-                                  const double* r, const double* e, const double* part, int nparts, long long stride,
-                                  float* G, float* c, float* d)
+                                  const double* r, const double* e, const double* part, int nparts, float* G,
+                                  float* c, float* d)
 {
     __shared__ double wgt;
     if (threadIdx.x == 0) {
@@ -103,61 +102,37 @@ __global__ void k_pair_accumulate(const int* rowptr, const int* col, const signe
         float rv[7] = {0, 0, 0, 0, 0, 0, 0};
         for (int p = rowptr[i]; p < rowptr[i + 1]; p++) rv[slot[p]] = (float)r[col[p]];
         const float ei = (float)e[i];
-#pragma unroll
         for (int k = 0; k < 7; k++) {
             const float wr = w * rv[k];
-            for (int l = k; l < 7; l++) G[spai_sym(k, l) * stride + i] += wr * rv[l];   // (symmetric)
-            c[k * stride + i] += wr * ei;
+            for (int l = 0; l < 7; l++) G[i * 49 + k * 7 + l] += wr * rv[l];
+            c[i * 7 + k] += wr * ei;
         }
         d[i] += w * ei * ei;
     }
 }
 
-// Adam on the FP32 master weights, with the weight image the network computes with
-struct AdamArgs {
-    float* master;
-    unsigned char* image;
-    float *m1, *m2;
-    int step;
-    float lr, b1, b2, eps;
-};
-__device__ __forceinline__ void adam_update(const AdamArgs& a, int i, float g)
-{
-    const float u = a.b1 * a.m1[i] + (1.f - a.b1) * g;
-    const float v = a.b2 * a.m2[i] + (1.f - a.b2) * g * g;
-    a.m1[i] = u;
-    a.m2[i] = v;
-    const float uh = u / (1.f - powf(a.b1, (float)a.step));
-    const float vh = v / (1.f - powf(a.b2, (float)a.step));
-    const float w = a.master[i] - a.lr * uh / (sqrtf(vh) + a.eps);
-    a.master[i] = w;
-    mlp_pack(a.image, i, w);
-}
-
-// Sum over the CTAs' partials gpart[b][idx] in FP64, then the Adam update (ADAM) or grad[idx].
-// Block x covers the 32 parameters 32x .. 32x+31 (one per lane, coalesced rows of gpart); its
-// eight warps take the partials b = w, w + 8, ... (ten loads in flight per lane), and the warps'
-// sums are added in warp order: a fixed order for a given nblk.
+// grad[idx] = sum over the CTAs' partials gpart[b][idx] in FP64.  Block x covers the 32
+// parameters 32x .. 32x+31 (one per lane, coalesced rows of gpart); its eight warps take
+// the partials b = w, w + 8, ... (eight loads in flight per lane), and the warps' sums are
+// added in warp order: a fixed order for a given nblk.
 constexpr int GR_THREADS = 256;
-template <bool ADAM>
-__global__ void __launch_bounds__(GR_THREADS) k_grad_reduce(const float* gpart, int nblk, double* grad, AdamArgs ad)
+__global__ void __launch_bounds__(GR_THREADS) k_grad_reduce(const float* gpart, int nblk, double* grad)
 {
-    constexpr int GW = GR_THREADS / 32, U = 10;
-    __shared__ double part[GW][32];
+    __shared__ double part[GR_THREADS / 32][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int idx = blockIdx.x * 32 + lane;
     double t = 0.0;
     if (idx < NPARAM) {
-        for (int b0 = warp; b0 < nblk; b0 += U * GW) {
-            float v[U];
+        for (int b0 = warp; b0 < nblk; b0 += 8 * (GR_THREADS / 32)) {
+            float v[8];
 #pragma unroll
-            for (int u = 0; u < U; u++) {
-                const int b = b0 + u * GW;
+            for (int u = 0; u < 8; u++) {
+                const int b = b0 + u * (GR_THREADS / 32);
                 v[u] = b < nblk ? gpart[(long long)b * NPARAM + idx] : 0.f;
             }
 #pragma unroll
-            for (int u = 0; u < U; u++)
-                if (b0 + u * GW < nblk) t = __dadd_rn(t, f32_to_f64_exact(v[u]));
+            for (int u = 0; u < 8; u++)
+                if (b0 + u * (GR_THREADS / 32) < nblk) t = __dadd_rn(t, f32_to_f64_exact(v[u]));
         }
     }
     part[warp][lane] = t;
@@ -165,16 +140,33 @@ __global__ void __launch_bounds__(GR_THREADS) k_grad_reduce(const float* gpart, 
     if (warp == 0 && idx < NPARAM) {
         double s = 0.0;
 #pragma unroll
-        for (int w = 0; w < GW; w++) s = __dadd_rn(s, part[w][lane]);
-        if constexpr (ADAM) adam_update(ad, idx, (float)s);
-        else grad[idx] = s;
+        for (int w = 0; w < GR_THREADS / 32; w++) s = __dadd_rn(s, part[w][lane]);
+        grad[idx] = s;
     }
 }
 
-__global__ void k_pack_weights(const float* master, unsigned char* image)
+// Adam on the FP32 master weights; the BF16-rounded copy is what the network computes with
+__global__ void k_adam(float* master, float* bf, const double* grad, float* m1, float* m2, int step, float lr,
+                       float b1, float b2, float eps)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NPARAM; i += gridDim.x * blockDim.x) {
+        const float g = (float)grad[i];
+        const float a = b1 * m1[i] + (1.f - b1) * g;
+        const float v = b2 * m2[i] + (1.f - b2) * g * g;
+        m1[i] = a;
+        m2[i] = v;
+        const float ah = a / (1.f - powf(b1, (float)step));
+        const float vh = v / (1.f - powf(b2, (float)step));
+        const float w = master[i] - lr * ah / (sqrtf(vh) + eps);
+        master[i] = w;
+        bf[i] = __bfloat162float(__float2bfloat16_rn(w));
+    }
+}
+
+__global__ void k_round_bf16(const float* master, float* bf)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NPARAM; i += gridDim.x * blockDim.x)
-        mlp_pack(image, i, master[i]);
+        bf[i] = __bfloat162float(__float2bfloat16_rn(master[i]));
 }
 
 __global__ void k_spai_pvals(const int* rowptr, const signed char* slot, long long n, const float* out,
@@ -199,14 +191,12 @@ struct cbg_spai {
     unsigned char* mask = nullptr;
     float* feat = nullptr;
     double* diag = nullptr;
-    float* idiag = nullptr;       // 1 / a_ii in FP32
-    long long stride = 0;         // rows between the arrays of G and c
     float *G = nullptr, *c = nullptr, *d = nullptr;
     double *e = nullptr, *r = nullptr, *part = nullptr;
-    unsigned char* image = nullptr;   // the weights as the network kernel reads them
-    float *master = nullptr, *m1 = nullptr, *m2 = nullptr, *out = nullptr;
+    float *master = nullptr, *bf = nullptr, *m1 = nullptr, *m2 = nullptr, *out = nullptr;
     float* gpart = nullptr;       // per-CTA gradient partials of the network kernel
     double* lpart = nullptr;      // per-CTA loss partials
+    double* grad = nullptr;
     int* fault = nullptr;         // a tensor-core wait ran out
     int tc_grid = 0;
     long long npairs = 0;
@@ -218,8 +208,8 @@ namespace {
 void free_spai(cbg_spai* s)
 {
     if (!s) return;
-    void* ps[] = {s->rowptr, s->col, s->val, s->slot, s->mask, s->feat, s->diag, s->idiag, s->G, s->c, s->d, s->e, s->r,
-                  s->part, s->master, s->image, s->m1, s->m2, s->out, s->gpart, s->lpart, s->fault};
+    void* ps[] = {s->rowptr, s->col, s->val, s->slot, s->mask, s->feat, s->diag, s->G, s->c, s->d, s->e, s->r,
+                  s->part, s->master, s->bf, s->m1, s->m2, s->out, s->gpart, s->lpart, s->grad, s->fault};
     for (void* p : ps) cudaFree(p);
     delete s;
 }
@@ -264,12 +254,11 @@ MlpArgs net_args(const cbg_spai* s)
     MlpArgs a{};
     a.n = s->n;
     a.feat = s->feat;
-    a.image = s->image;
+    a.params = s->bf;
     a.G = s->G;
     a.c = s->c;
     a.d = s->d;
-    a.idiag = s->idiag;
-    a.stride = s->stride;
+    a.diag = s->diag;
     a.mask = s->mask;
     a.inv_npairs = 1.0 / (double)std::max<long long>(1, s->npairs);
     a.gpart = s->gpart;
@@ -286,7 +275,7 @@ int train_pass(cbg_spai* s, double* loss)
     if (rc || !loss) return rc;
     std::vector<double> parts(s->tc_grid);
     int fault = 0;
-    rc = check(cudaMemcpyAsync(parts.data(), s->lpart, parts.size() * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+    rc = check(cudaMemcpyAsync(parts.data(), s->lpart, s->tc_grid * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
     if (!rc) rc = check(cudaMemcpyAsync(&fault, s->fault, sizeof(int), cudaMemcpyDeviceToHost, s->stream));
     if (!rc) rc = check(cudaStreamSynchronize(s->stream));
     if (rc) return rc;
@@ -330,22 +319,19 @@ int cbg_spai_create(const cbg_csr* A, int64_t sx, int64_t sxy, const cbg_options
     TRY(check(cudaMemcpy(s->col, A->col, nnz * sizeof(int), k)));
     TRY(check(cudaMemcpy(s->val, A->val, nnz * sizeof(double), k)));
     TRY(alloc(&s->slot, nnz)); TRY(alloc(&s->mask, np)); TRY(alloc(&s->feat, np * NIN)); TRY(alloc(&s->diag, np));
-    TRY(alloc(&s->idiag, np));
-    s->stride = np;
-    TRY(alloc(&s->G, np * 28)); TRY(alloc(&s->c, np * 7)); TRY(alloc(&s->d, np));
+    TRY(alloc(&s->G, np * 49)); TRY(alloc(&s->c, np * 7)); TRY(alloc(&s->d, np));
     TRY(alloc(&s->e, n)); TRY(alloc(&s->r, n)); TRY(alloc(&s->part, 4096));
-    TRY(alloc(&s->master, NPARAM)); TRY(alloc(&s->image, MLP_IMAGE)); TRY(alloc(&s->m1, NPARAM)); TRY(alloc(&s->m2, NPARAM));
-    TRY(alloc(&s->out, np * NOUT)); TRY(alloc(&s->fault, 1));
+    TRY(alloc(&s->master, NPARAM)); TRY(alloc(&s->bf, NPARAM)); TRY(alloc(&s->m1, NPARAM)); TRY(alloc(&s->m2, NPARAM));
+    TRY(alloc(&s->out, np * NOUT)); TRY(alloc(&s->grad, NPARAM)); TRY(alloc(&s->fault, 1));
     s->tc_grid = mlp_tc_grid(n);
     TRY(alloc(&s->gpart, (size_t)s->tc_grid * NPARAM));
     TRY(alloc(&s->lpart, (size_t)s->tc_grid));
-    TRY(check(cudaMemset(s->G, 0, np * 28 * sizeof(float))));
+    TRY(check(cudaMemset(s->G, 0, np * 49 * sizeof(float))));
     TRY(check(cudaMemset(s->c, 0, np * 7 * sizeof(float))));
     TRY(check(cudaMemset(s->d, 0, np * sizeof(float))));
     TRY(check(cudaMemset(s->mask, 0, np)));
     TRY(check(cudaMemset(s->feat, 0, np * NIN * sizeof(float))));
     TRY(check(cudaMemset(s->fault, 0, sizeof(int))));
-    TRY(check(cudaMemset(s->image, 0, MLP_IMAGE)));
     if (np > n) {
         std::vector<double> ones(np - n, 1.0);
         TRY(check(cudaMemcpy(s->diag + n, ones.data(), (np - n) * sizeof(double), cudaMemcpyHostToDevice)));
@@ -354,15 +340,14 @@ int cbg_spai_create(const cbg_csr* A, int64_t sx, int64_t sxy, const cbg_options
     TRY(check(cudaMemset(s->m2, 0, NPARAM * sizeof(float))));
     int* bad = reinterpret_cast<int*>(s->part);
     TRY(check(cudaMemset(bad, 0, sizeof(int))));
-    k_spai_setup<<<grid_rows(n), LT>>>(s->rowptr, s->col, s->val, n, sx, sxy, s->slot, s->feat, s->diag, s->idiag, s->mask,
-                                      bad);
+    k_spai_setup<<<grid_rows(n), LT>>>(s->rowptr, s->col, s->val, n, sx, sxy, s->slot, s->feat, s->diag, s->mask, bad);
     int hbad = 0;
     TRY(check(cudaMemcpy(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost)));
     if (hbad) TRY(CBG_ERR_ARG);   // not a 7-point pattern with these strides, or a zero diagonal
     std::vector<float> w;
     init_params(w, 20201201ull);
     TRY(check(cudaMemcpy(s->master, w.data(), NPARAM * sizeof(float), cudaMemcpyHostToDevice)));
-    k_pack_weights<<<32, 256>>>(s->master, s->image);
+    k_round_bf16<<<32, 256>>>(s->master, s->bf);
     TRY(check(cudaDeviceSynchronize()));
 #undef TRY
     *out = s;
@@ -374,8 +359,8 @@ int cbg_spai_add_pair(cbg_spai* s, const double* xstar, const double* xk)
     if (!s || !xstar || !xk) return CBG_ERR_ARG;
     const int g = grid_rows(s->n);
     k_pair_residual<<<g, LT, 0, s->stream>>>(s->rowptr, s->col, s->val, s->n, xstar, xk, s->e, s->r, s->part);
-    k_pair_accumulate<<<g, LT, 0, s->stream>>>(s->rowptr, s->col, s->slot, s->n, s->r, s->e, s->part, g, s->stride, s->G,
-                                              s->c, s->d);
+    k_pair_accumulate<<<g, LT, 0, s->stream>>>(s->rowptr, s->col, s->slot, s->n, s->r, s->e, s->part, g, s->G, s->c,
+                                              s->d);
     int rc = check(cudaGetLastError());
     if (!rc) s->npairs++;
     return rc;
@@ -395,9 +380,10 @@ int cbg_spai_train(cbg_spai* s, int steps, double lr, double* loss_first, double
         // the loss is read back once, before the first update (no per-step synchronisation)
         int rc = train_pass(s, it == 0 ? &l0 : nullptr);
         if (rc) return rc;
+        k_grad_reduce<<<(NPARAM + 31) / 32, GR_THREADS, 0, s->stream>>>(s->gpart, s->tc_grid, s->grad);
         s->step++;
-        const AdamArgs ad{s->master, s->image, s->m1, s->m2, s->step, (float)lr, 0.9f, 0.999f, 1e-8f};
-        k_grad_reduce<true><<<(NPARAM + 31) / 32, GR_THREADS, 0, s->stream>>>(s->gpart, s->tc_grid, nullptr, ad);
+        k_adam<<<(NPARAM + 255) / 256, 256, 0, s->stream>>>(s->master, s->bf, s->grad, s->m1, s->m2, s->step,
+                                                            (float)lr, 0.9f, 0.999f, 1e-8f);
         rc = check(cudaGetLastError());
         if (rc) return rc;
     }
@@ -429,7 +415,7 @@ int cbg_spai_params(cbg_spai* s, float* params, int set)
     if (set) {
         int rc = check(cudaMemcpy(s->master, params, NPARAM * sizeof(float), cudaMemcpyHostToDevice));
         if (rc) return rc;
-        k_pack_weights<<<32, 256, 0, s->stream>>>(s->master, s->image);
+        k_round_bf16<<<32, 256, 0, s->stream>>>(s->master, s->bf);
         return check(cudaStreamSynchronize(s->stream));
     }
     return check(cudaMemcpy(params, s->master, NPARAM * sizeof(float), cudaMemcpyDeviceToHost));
@@ -449,21 +435,19 @@ int cbg_mlp_forward(int64_t rows, const float* feat, const float* params_host, f
 {
     if (rows < 1 || !feat || !params_host || !out || ((uintptr_t)feat & 15)) return CBG_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
-    float* m = nullptr;
-    unsigned char* b = nullptr;
+    float *m = nullptr, *b = nullptr;
     int* fault = nullptr;
     int rc = alloc(&m, NPARAM);
-    if (!rc) rc = alloc(&b, MLP_IMAGE);
-    if (!rc) rc = check(cudaMemsetAsync(b, 0, MLP_IMAGE, st));
+    if (!rc) rc = alloc(&b, NPARAM);
     if (!rc) rc = alloc(&fault, 1);
     if (!rc) rc = check(cudaMemsetAsync(fault, 0, sizeof(int), st));
     if (!rc) rc = check(cudaMemcpyAsync(m, params_host, NPARAM * sizeof(float), cudaMemcpyHostToDevice, st));
     if (!rc) {
-        k_pack_weights<<<32, 256, 0, st>>>(m, b);
+        k_round_bf16<<<32, 256, 0, st>>>(m, b);
         MlpArgs a{};
         a.n = rows;
         a.feat = feat;
-        a.image = b;
+        a.params = b;
         a.out = out;
         a.fault = fault;
         rc = check(mlp_tc_launch(MLP_FWD, mlp_tc_grid(rows), st, a));
@@ -485,30 +469,28 @@ int cbg_mlp_backward(int64_t rows, const float* feat, const float* params_host, 
         return CBG_ERR_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     const int grid = mlp_tc_grid(rows);
-    float *m = nullptr, *gp = nullptr;
-    unsigned char* b = nullptr;
+    float *m = nullptr, *b = nullptr, *gp = nullptr;
     double* g = nullptr;
     int* fault = nullptr;
     int rc = alloc(&m, NPARAM);
-    if (!rc) rc = alloc(&b, MLP_IMAGE);
-    if (!rc) rc = check(cudaMemsetAsync(b, 0, MLP_IMAGE, st));
+    if (!rc) rc = alloc(&b, NPARAM);
     if (!rc) rc = alloc(&gp, (size_t)grid * NPARAM);
     if (!rc) rc = alloc(&g, NPARAM);
     if (!rc) rc = alloc(&fault, 1);
     if (!rc) rc = check(cudaMemsetAsync(fault, 0, sizeof(int), st));
     if (!rc) rc = check(cudaMemcpyAsync(m, params_host, NPARAM * sizeof(float), cudaMemcpyHostToDevice, st));
     if (!rc) {
-        k_pack_weights<<<32, 256, 0, st>>>(m, b);
+        k_round_bf16<<<32, 256, 0, st>>>(m, b);
         MlpArgs a{};
         a.n = rows;
         a.feat = feat;
-        a.image = b;
+        a.params = b;
         a.gout = gout;
         a.gpart = gp;
         a.fault = fault;
         rc = check(mlp_tc_launch(MLP_BWD, grid, st, a));
         if (!rc) {
-            k_grad_reduce<false><<<(NPARAM + 31) / 32, GR_THREADS, 0, st>>>(gp, grid, g, AdamArgs{});
+            k_grad_reduce<<<(NPARAM + 31) / 32, GR_THREADS, 0, st>>>(gp, grid, g);
             rc = check(cudaGetLastError());
         }
         int hf = 0;
