@@ -286,6 +286,11 @@ template <int FMT> struct BatchedSolver {
         return df_to_double(ssS, ssC);
     }
 
+    // End of the chunks r0 >> 5, ... of a block's rows [r0, r1).  A block's rows start at a multiple
+    // of 32, except that a trailing rank of a cluster may own none (r0 = r1 = n): its r0 may lie
+    // inside the last chunk, which belongs to another block.
+    static __device__ __forceinline__ int sell_end(int r0, int r1) { return r1 > r0 ? (r1 + 31) >> 5 : r0 >> 5; }
+
     // spmv_df on the sliced-ELL planes: a warp takes four chunks of 32 rows at a time (a lane
     // per row), every load of columns and values is one contiguous 128-byte access, and the next
     // entries are loaded while the current ones' gathers are in flight.
@@ -302,7 +307,7 @@ template <int FMT> struct BatchedSolver {
         float xsh = 1.f, xsl = 0.f;
         if (xsplit) split_f64(xscale, xsh, xsl);
         float ssS = 0.f, ssC = 0.f;
-        const int cb = r0 >> 5, ce = (r1 + 31) >> 5;               // (r0 is a multiple of 32)
+        const int cb = r0 >> 5, ce = sell_end(r0, r1);
         for (int c0 = cb + warp * RW; c0 < ce; c0 += NW * RW) {
             float S[RW], C[RW], vh[RW], vl[RW];
             long long p[RW];
@@ -380,7 +385,7 @@ template <int FMT> struct BatchedSolver {
         float* wl = sm->w + a.max_rows_block;
         const long long* off = a.sell_off + s.ch_off;
         double ss = 0.0;
-        const int cb = r0 >> 5, ce = (r1 + 31) >> 5;
+        const int cb = r0 >> 5, ce = sell_end(r0, r1);
         for (int c0 = cb + warp * RW; c0 < ce; c0 += NW * RW) {
             double t[RW], v[RW];
             long long p[RW];
