@@ -279,7 +279,8 @@ int cbg_basis_axpy(int fmt, int arith, int64_t n, int ncols, const void* V, int6
  * smaller); each group reads V once for all its vectors (one split-K product in
  * double-float arithmetic, like cbg_basis_dot with arith = CBG_ARITH_DF32).
  *   V: device codes of format fmt, ncols (<= 320) columns of leading dimension ld
- *      elements (ld >= n, ld % 4096 == 0, rows n..ld-1 zero);
+ *      elements (ld >= n, ld % 4096 == 0, rows n..ld-1 zero), at any address aligned to
+ *      its code type (fastest from a 16-byte boundary; the tensor cores need one);
  *   scales[ncols]: device decode factors;  W: device, n x k column-major, leading
  *      dimension ldw >= n (only rows < n are read);
  *   H: device, ncols x k row-major: H[c*k + r] = sum_i dec(V[i,c]) W[i,r];
@@ -293,7 +294,8 @@ int cbg_basis_dot_multi(int fmt, int64_t n, int ncols, const void* V, int64_t ld
                         void* stream);
 /* The same product with the implementation chosen by `path`: 0 automatic (what
  * cbg_basis_dot_multi does), 1 CUDA cores (double-float, every format), 2 tensor cores
- * (tcgen05, f16 basis with ncols <= 128, else CBG_ERR_UNSUPPORTED).  The tensor-core
+ * (tcgen05, f16 basis with ncols <= 128 on a 16-byte boundary, else
+ * CBG_ERR_UNSUPPORTED; automatic takes the CUDA cores then).  The tensor-core
  * path cuts codes and vectors into small pieces whose FP16 products and FP32 sums are
  * exact; W is truncated once, 54 bits below the largest |W| of each 512-row block, so
  * H matches the double-float path to FP64-level accuracy.  It covers codes with

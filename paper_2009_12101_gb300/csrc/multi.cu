@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "../../include/cbgmres.h"
 #include "cbg_kernels.cuh"
@@ -48,6 +49,8 @@ constexpr int MU_CPW = 2;            // columns per consumer warp
 constexpr int MU_CG = MU_CS * MU_CPW;   // columns per stage
 constexpr int MU_THREADS = (MU_CW + 1) * 32;
 constexpr int MU_CHAIN = 32;         // rows a lane accumulates before its sums are folded (one pair of vectors: half)
+
+__host__ __device__ inline bool aligned16(const void* p) { return (reinterpret_cast<size_t>(p) & 15) == 0; }
 
 template <int FMT, int KP> struct MultiGeom {
     static constexpr int BS = FmtInfo<FMT>::bytes;
@@ -99,9 +102,24 @@ __global__ void k_split_multi(const double* W, long long ldw, long long n, long 
     }
 }
 
+// Sixteen bytes of codes of BS bytes each, read one by one: a basis that starts between 16-byte
+// boundaries, which neither the bulk copies nor 16-byte loads can take.
+template <int BS> __device__ __forceinline__ uint4 load_codes(const unsigned char* p)
+{
+    using T = typename std::conditional<BS == 8, unsigned long long,
+              typename std::conditional<BS == 4, unsigned int,
+              typename std::conditional<BS == 2, unsigned short, unsigned char>::type>::type>::type;
+    union { T c[16 / BS]; uint4 v; } u;
+#pragma unroll
+    for (int e = 0; e < 16 / BS; e++) u.c[e] = reinterpret_cast<const T*>(p)[e];
+    return u.v;
+}
+
 __device__ __forceinline__ void multi_sync() { asm volatile("bar.sync 1, %0;" ::"r"(MU_CW * 32) : "memory"); }
 
-template <int FMT, int KP>
+// DIRECT: the basis is not on a 16-byte boundary, the consumers read its codes themselves
+// (a branch at run time in place of the parameter made the aligned kernels spill)
+template <int FMT, int KP, bool DIRECT>
 __global__ void __launch_bounds__(MU_THREADS, 1) k_dot_multi(MultiArgs a, int stages)
 {
     using G = MultiGeom<FMT, KP>;
@@ -141,9 +159,9 @@ __global__ void __launch_bounds__(MU_THREADS, 1) k_dot_multi(MultiArgs a, int st
             const int c0 = g * MU_CG, nc = a.ncols - c0 < MU_CG ? a.ncols - c0 : MU_CG;
             if (it >= stages && !warp_wait(&empty[rg.s], rg.ph ^ 1u)) { failed = 1; break; }
             unsigned char* st = mu_ring + (size_t)rg.s * G::STAGE;
-            if (lane == 0) mbar_arrive_expect_tx(&full[rg.s], (unsigned)(nc * G::COLB + 2 * KP * G::PLANE));
+            if (lane == 0) mbar_arrive_expect_tx(&full[rg.s], (unsigned)((DIRECT ? 0 : nc * G::COLB) + 2 * KP * G::PLANE));
             __syncwarp();
-            if (lane < nc)
+            if (!DIRECT && lane < nc)
                 bulk_g2s_hint(st + lane * G::COLB, a.V + (long long)(c0 + lane) * a.ldb + t * G::COLB, G::COLB, &full[rg.s], pol);
             if (lane >= 16 && lane < 16 + 2 * KP)
                 bulk_g2s(st + MU_CG * G::COLB + (lane - 16) * G::PLANE, a.wsplit + (lane - 16) * a.ld + t * G::TILE, G::PLANE,
@@ -204,8 +222,13 @@ __global__ void __launch_bounds__(MU_THREADS, 1) k_dot_multi(MultiArgs a, int st
                     if (q0 < nc) {                    // (a missing column's stale codes are never read back)
                         Chunk<FMT> ch[MU_CPW];
 #pragma unroll
-                        for (int q = 0; q < MU_CPW; q++)
-                            decode_chunk<FMT>(*reinterpret_cast<const uint4*>(st + (q0 + q) * G::COLB + ln * 16), ch[q]);
+                        for (int q = 0; q < MU_CPW; q++) {
+                            uint4 raw = make_uint4(0u, 0u, 0u, 0u);
+                            if (!DIRECT) raw = *reinterpret_cast<const uint4*>(st + (q0 + q) * G::COLB + ln * 16);
+                            else if (q0 + q < nc)
+                                raw = load_codes<G::BS>(a.V + (long long)(c0 + q0 + q) * a.ldb + t * G::COLB + ln * 16);
+                            decode_chunk<FMT>(raw, ch[q]);
+                        }
                         const float4* wt = reinterpret_cast<const float4*>(st + MU_CG * G::COLB) + ln;
 #pragma unroll
                         for (int e = 0; e < E; e += 2) {
@@ -295,19 +318,25 @@ __global__ void __launch_bounds__(256) k_multi_sum(const double* part, int nblk,
     }
 }
 
-template <int FMT, int KP> void launch_multi(int grid, cudaStream_t s, const MultiArgs& a)
+template <int FMT, int KP, bool DIRECT> void launch_multi(int grid, cudaStream_t s, const MultiArgs& a)
 {
     using G = MultiGeom<FMT, KP>;
     static const int stages = [] {
         cudaFuncAttributes fa{};
-        const int st = cudaFuncGetAttributes(&fa, k_dot_multi<FMT, KP>) == cudaSuccess
+        const int st = cudaFuncGetAttributes(&fa, k_dot_multi<FMT, KP, DIRECT>) == cudaSuccess
                            ? tma_stages(G::STAGE, (int)fa.sharedSizeBytes) : 0;
         if (st >= 2)
-            cudaFuncSetAttribute(k_dot_multi<FMT, KP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            cudaFuncSetAttribute(k_dot_multi<FMT, KP, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)tma_smem_bytes(st, G::STAGE));
         return st;
     }();
-    k_dot_multi<FMT, KP><<<grid, MU_THREADS, tma_smem_bytes(stages, G::STAGE), s>>>(a, stages);
+    k_dot_multi<FMT, KP, DIRECT><<<grid, MU_THREADS, tma_smem_bytes(stages, G::STAGE), s>>>(a, stages);
+}
+
+template <int FMT, int KP> void launch_multi(int grid, cudaStream_t s, const MultiArgs& a)
+{
+    if (aligned16(a.V)) launch_multi<FMT, KP, false>(grid, s, a);
+    else launch_multi<FMT, KP, true>(grid, s, a);
 }
 
 template <int KP> void launch_fmt(int fmt, int grid, cudaStream_t s, const MultiArgs& a)
@@ -341,11 +370,14 @@ int dot_multi_group(int fmt, int64_t n, int ncols, const void* V, int64_t ld, co
         return CBG_OK;
     }
     const int KP = (k + 1) / 2, grid = multi_grid();
+    // [fault word | planes of W | partials], the planes on the last 16-byte boundary of the first 256
+    // bytes' end (the workspace itself may lie anywhere)
     unsigned char* ws = static_cast<unsigned char*>(workspace);
-    int* fault = reinterpret_cast<int*>(ws);
-    float2* wsplit = reinterpret_cast<float2*>(ws + 256);
+    ws += 256 - (reinterpret_cast<size_t>(ws) & 15);
+    int* fault = reinterpret_cast<int*>(ws - 16);
+    float2* wsplit = reinterpret_cast<float2*>(ws);
     const size_t split = (size_t)2 * KP * ld * sizeof(float2);
-    double* part = reinterpret_cast<double*>(ws + 256 + (split + 255) / 256 * 256);
+    double* part = reinterpret_cast<double*>(ws + (split + 255) / 256 * 256);
     const int E = 16 / cbgmres_format_bytes(fmt);
     k_split_multi<<<(int)std::min<long long>(((long long)KP * ld / 2 + 255) / 256, 4096), 256, 0, s>>>(
         W, ldw, n, ld, k, KP, E, wsplit, fault);
@@ -390,7 +422,7 @@ int cbg_basis_dot_multi_path(int fmt, int64_t n, int ncols, const void* V, int64
         ws_bytes < cbg_basis_dot_multi_workspace(ld, ncols, k) || path < 0 || path > 2)
         return CBG_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const bool tc_ok = fmt == CBG_F16 && ncols <= 128;
+    const bool tc_ok = fmt == CBG_F16 && ncols <= 128 && aligned16(V);   // (it reads 16 bytes at a time)
     if (path == 2 && !tc_ok) return CBG_ERR_UNSUPPORTED;
     const bool tc = path == 2 || (path == 0 && tc_ok);
     // groups of up to KMAX vectors, one after the other on the stream (the workspace is reused)
