@@ -89,7 +89,7 @@ struct BtSmem {
     double red[BT_MAXM + 4];           // this block's partial sums (read by the cluster)
     double tot[BT_MAXM + 4];           // team totals
     double wred[BT_THREADS / 32][BT_MAXM + 4];   // (the dot: row splits' sums as float2)
-    double hn, inv, omega;             // of the current step (formed by one thread: an FP64 instruction
+    double inv, omega;                 // of the current step (formed by one thread: an FP64 instruction
     EncParams ep;                      // occupies the narrow pipe for a whole warp)
     int sys_idx;
     int stop;
@@ -535,6 +535,13 @@ template <int FMT> struct BatchedSolver {
         return df_to_double(ssS, ssC);
     }
 
+    // 16 bytes of codes.  encode() writes the columns in this launch, and again in every cycle, so
+    // the loads are coherent ones past L1 (ld.global.nc is for data that no one writes).
+    static __device__ __forceinline__ uint4 codes16(const unsigned char* p)
+    {
+        return __ldcg(reinterpret_cast<const uint4*>(p));
+    }
+
     // partial h_k = sum over own rows of dec(V_k) w, k < ncols, into sm->red[0..ncols) (scale
     // applied).  Warps are dealt out as row splits x groups of eight columns so that the
     // slowest has the fewest (group, segment of 32 chunks) items; a warp reads its rows of w
@@ -572,7 +579,7 @@ template <int FMT> struct BatchedSolver {
                 const unsigned char* p = vc + (long long)q0 * vstride + ch * 16;
 #pragma unroll
                 for (int q = 0; q < H; q++) {
-                    raw[q] = ch < nch && q0 + q < nc ? ldg_stream(p) : make_uint4(0u, 0u, 0u, 0u);
+                    raw[q] = ch < nch && q0 + q < nc ? codes16(p) : make_uint4(0u, 0u, 0u, 0u);
                     p += vstride;
                 }
             };
@@ -669,7 +676,7 @@ template <int FMT> struct BatchedSolver {
                 const unsigned char* p = cp + (long long)k0 * vstride;
 #pragma unroll
                 for (int q = 0; q < U; q++) {
-                    raw[q] = in && k0 + q * ks < ncols ? ldg_stream(p) : make_uint4(0u, 0u, 0u, 0u);
+                    raw[q] = in && k0 + q * ks < ncols ? codes16(p) : make_uint4(0u, 0u, 0u, 0u);
                     p += ks * vstride;
                 }
             };
