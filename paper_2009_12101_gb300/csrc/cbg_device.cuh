@@ -525,20 +525,54 @@ __device__ __forceinline__ void df_warp_sum(float& S, float& C)
     }
 }
 
-// The block's double-float sum of the threads' (S, C); valid in warp 0.  red: shared, one entry
-// per warp.  All threads call it.
-__device__ __forceinline__ float2 df_block_sum(float S, float C, float2* red)
+// Sums of FP32 pairs across threads, warps and blocks without loss against FP64 additions and
+// without the FP64 pipe: three floats x + y + z.  x and y take the sum and its rounding errors by
+// two_sum, z what remains of those, so an addition loses about 2^-70 of the sum (FP64: 2^-53; an
+// addition of pairs 2^-46).  The first two two_sums are independent: the chain through an addition
+// is as long as that of pairs.
+__device__ __forceinline__ void tf_add(float4& a, float h, float l, float z = 0.f)
+{
+    float e, t, f, g;
+    two_sum(a.x, h, a.x, e);
+    two_sum(a.y, l, t, f);
+    two_sum(t, e, a.y, g);
+    a.z = __fadd_rn(__fadd_rn(a.z, z), __fadd_rn(f, g));
+}
+__device__ __forceinline__ void tf_add(float4& a, const float4& b) { tf_add(a, b.x, b.y, b.z); }
+__device__ __forceinline__ double tf_to_double(const float4& a)
+{
+    return __dadd_rn((double)a.x, __dadd_rn((double)a.y, (double)a.z));
+}
+__device__ __forceinline__ float4 tf_shfl_xor(const float4& a, int o)
+{
+    return make_float4(__shfl_xor_sync(0xFFFFFFFFu, a.x, o), __shfl_xor_sync(0xFFFFFFFFu, a.y, o),
+                       __shfl_xor_sync(0xFFFFFFFFu, a.z, o), 0.f);
+}
+// (every lane holds the result).  Loops, here and in what uses it: a kernel's tail runs once, and
+// instructions that are fetched for a single use cost more than those that run (written out, the
+// tails of the axpy and of the one-pass kernel took 1 to 3 us longer).
+__device__ __forceinline__ void tf_warp_sum(float4& a)
+{
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) tf_add(a, tf_shfl_xor(a, o));
+}
+
+// The block's sum of the threads' a; valid in warp 0.  red: shared, one entry per warp.  All threads
+// call it.
+__device__ __forceinline__ float4 tf_block_sum(float4 a, float4* red)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    df_warp_sum(S, C);
-    if (lane == 0) red[warp] = make_float2(S, C);
-    __syncthreads();
-    float2 t = make_float2(0.f, 0.f);
-    if (warp == 0) {
-        if (lane < nw) t = red[lane];
-        df_warp_sum(t.x, t.y);
+#pragma unroll 1
+    for (int round = 0; round < 2; round++) {            // the warps, then warp 0 over their sums
+        tf_warp_sum(a);
+        if (round == 0) {
+            if (lane == 0) red[warp] = a;
+            __syncthreads();
+            if (warp != 0) break;
+            a = lane < nw ? red[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     }
-    return t;
+    return a;
 }
 
 // maximum of non-negative doubles over the warp, compared as bit patterns with 32-bit

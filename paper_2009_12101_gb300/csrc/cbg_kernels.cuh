@@ -62,7 +62,7 @@ struct DevArrays {
     double* scales;       // decode scale per basis column [m+1]
     double* hist;         // recurrence residual history (device)
     double* part;         // per-block partial sums [gridmax * (m+2)]
-    double* part_norm;    // per-block (sum of squares, max) of the axpy epilogue [gridmax*2]
+    double* part_norm;    // per-block (sum of squares, max) of the axpy epilogue [gridmax*4]
     double* part_spmv;    // per-block sum of squares and max of SpMV / residual [gridmax*2]
     unsigned int* counters;   // last-block counters (zeroed, reset by the last block)
     int* flag_host;       // mapped host copy of `active` (may be null)
@@ -138,24 +138,25 @@ __device__ __forceinline__ void block_reduce_norm_parts(const double* part, int 
     block_sum_max(s, __hiloint2double((int)mh, (int)ml), rs, rm, ss, mx);
 }
 
-// The last block's ||.|| from per-block double-float sums of squares part[b] (all threads call
-// it; valid in thread 0): thread t adds the pairs t, t + blockDim.x, ..., then a fixed tree.
-__device__ __forceinline__ double df_block_norm(const float2* part, int np)
+// The last block's ||.|| from the blocks' sums of squares part[b * step], b < np, as tf_add's triples
+// (all threads call it; valid in thread 0): thread t adds the triples t, t + blockDim.x, ..., then
+// a fixed tree.
+__device__ __forceinline__ double tf_block_norm(const float4* part, int step, int np)
 {
-    __shared__ float2 red[32];
-    float S = 0.f, C = 0.f;
+    __shared__ float4 red[32];
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int p0 = threadIdx.x; p0 < np; p0 += 4 * blockDim.x) {
-        float2 v[4];
+        float4 v[4];
 #pragma unroll
         for (int u = 0; u < 4; u++) {
             const int p = p0 + u * blockDim.x;
-            v[u] = p < np ? __ldcg(part + 2 * p) : make_float2(0.f, 0.f);
+            v[u] = p < np ? __ldcg(part + p * step) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int u = 0; u < 4; u++) df_add(S, C, v[u].x, v[u].y);
+        for (int u = 0; u < 4; u++) tf_add(s, v[u]);
     }
-    const float2 t = df_block_sum(S, C, red);
-    return threadIdx.x == 0 ? sqrt(df_to_double(t.x, t.y)) : 0.0;
+    s = tf_block_sum(s, red);
+    return threadIdx.x == 0 ? sqrt(tf_to_double(s)) : 0.0;
 }
 
 // The last block's sums over the per-block partials of nitems items: item i is
@@ -500,7 +501,7 @@ struct AxpyArgs {
     const double* dinv;       // Jacobi (EPI_XUPD), may be null
     long long nrows;          // ld
     long long n;              // true rows (norms exclude padding)
-    double* part_norm;        // [gridDim.x][2]
+    double* part_norm;        // [gridDim.x][4] (DF32: a triple of floats, the maximum; FP64: two doubles)
     const int* active;
     unsigned int* counter;    // EPI_SUB final pass: last block writes st->wnorm, st->wmax
     DevState* st;
@@ -720,25 +721,25 @@ __global__ void __launch_bounds__(THREADS, FmtInfo<FMT>::bytes >= 8 ? 4 : (FmtIn
     if constexpr (EPI == EPI_SUB) {
         if (!a.counter) return;
         if constexpr (ARITH == ARITH_DF32) {
-            // sums in double-float (with the dot's and the SpMV's: 2 % of a large solve, which
-            // the FP64 trees of every block spent on the narrow pipe)
-            __shared__ float2 red_df[THREADS / 32];
-            const float2 t = df_block_sum(ssS, ssC, red_df);
+            // sums as triples of floats (with the dot's and the SpMV's: 2 % of a large solve,
+            // which the FP64 trees of every block spent on the narrow pipe)
+            __shared__ float4 red_tf[THREADS / 32];
+            const float4 t = tf_block_sum(make_float4(ssS, ssC, 0.f, 0.f), red_tf);
             const double m0 = warp_max_nonneg(__hiloint2double((int)mxh, (int)mxl));
             if ((threadIdx.x & 31) == 0) red_m[threadIdx.x >> 5] = m0;
             __syncthreads();
             if (threadIdx.x < 32) {
                 const double m = warp_max_nonneg(threadIdx.x < THREADS / 32 ? red_m[threadIdx.x] : 0.0);
                 if (threadIdx.x == 0) {
-                    reinterpret_cast<float2*>(a.part_norm)[2 * blockIdx.x] = t;
-                    a.part_norm[2 * blockIdx.x + 1] = m;
+                    reinterpret_cast<float4*>(a.part_norm)[2 * blockIdx.x] = t;
+                    a.part_norm[4 * blockIdx.x + 2] = m;
                 }
             }
             if (last_block(a.counter)) {
-                const double wn = df_block_norm(reinterpret_cast<const float2*>(a.part_norm), gridDim.x);
+                const double wn = tf_block_norm(reinterpret_cast<const float4*>(a.part_norm), 2, gridDim.x);
                 unsigned int h = 0u, l = 0u;           // the maximum, on bit patterns
                 for (int p = threadIdx.x; p < gridDim.x; p += THREADS) {
-                    const double v = __ldcg(a.part_norm + 2 * p + 1);
+                    const double v = __ldcg(a.part_norm + 4 * p + 2);
                     const unsigned int vh = (unsigned int)__double2hiint(v), vl = (unsigned int)__double2loint(v);
                     if (vh > h || (vh == h && vl > l)) {
                         h = vh;
@@ -1152,12 +1153,12 @@ __global__ void __launch_bounds__(THREADS) k_spmv(SpmvArgs a)
     const double mx = __longlong_as_double((long long)mxb);
     if constexpr (MODE == SPMV_PLAIN || MODE == SPMV_ACCUM) return;
     else {
-        if (dfrows) {                        // omega of the double-float rows, summed in double-float
-            __shared__ float2 red_df[THREADS / 32];
-            const float2 t = df_block_sum(ssS, ssC, red_df);
-            if (threadIdx.x == 0) reinterpret_cast<float2*>(a.part)[2 * blockIdx.x] = t;
+        if (dfrows) {                        // omega of the double-float rows
+            __shared__ float4 red_tf[THREADS / 32];
+            const float4 t = tf_block_sum(make_float4(ssS, ssC, 0.f, 0.f), red_tf);
+            if (threadIdx.x == 0) reinterpret_cast<float4*>(a.part)[blockIdx.x] = t;
             if (last_block(a.counter)) {
-                const double om = df_block_norm(reinterpret_cast<const float2*>(a.part), gridDim.x);
+                const double om = tf_block_norm(reinterpret_cast<const float4*>(a.part), 1, gridDim.x);
                 if (threadIdx.x == 0) a.st->omega = om;
             }
             return;
@@ -1217,7 +1218,7 @@ template <int XFMT>
 __global__ void __launch_bounds__(THREADS) k_spmv_sell(SellArgs a)
 {
     if (a.active && *a.active == 0) return;
-    __shared__ float2 red_df[THREADS / 32];
+    __shared__ float4 red_tf[THREADS / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr bool XEXACT = XFMT == F32 || XFMT == F16 || XFMT == BF16 || XFMT == E4M3 || XFMT == I16;
     const double xs = a.xscale_dev ? *a.xscale_dev : 1.0;
@@ -1289,10 +1290,10 @@ __global__ void __launch_bounds__(THREADS) k_spmv_sell(SellArgs a)
             dfadd(ssS, ssC, p, e);
         }
     }
-    const float2 t = df_block_sum(ssS, ssC, red_df);
-    if (threadIdx.x == 0) reinterpret_cast<float2*>(a.part)[2 * blockIdx.x] = t;
+    const float4 t = tf_block_sum(make_float4(ssS, ssC, 0.f, 0.f), red_tf);
+    if (threadIdx.x == 0) reinterpret_cast<float4*>(a.part)[blockIdx.x] = t;
     if (last_block(a.counter)) {
-        const double om = df_block_norm(reinterpret_cast<const float2*>(a.part), gridDim.x);
+        const double om = tf_block_norm(reinterpret_cast<const float4*>(a.part), 1, gridDim.x);
         if (threadIdx.x == 0) a.st->omega = om;
     }
 }

@@ -209,39 +209,35 @@ __device__ __forceinline__ void consumers_sync()
     asm volatile("bar.sync 1, %0;" ::"r"(DOT_CW * 32) : "memory");
 }
 
-// The blocks' column totals tot (shared memory, written by all threads before) to
+// The blocks' column totals (a.part[block][MAXCOLS], written by the block's threads before) to
 // a.out = scales .* total.  Grid barrier (the kernels are launched cooperatively: every block
 // is resident), then block b adds the partials of the columns b, b + gridDim.x, ..., a warp per
 // column: its lanes add the blocks lane, lane + 32, ... (five loads in flight) and fold.  The
-// cross-block sum is spread over all SMs, and in double-float: an FP64 instruction occupies
-// GB300's pipe for 20 cycles per SM, and the FP64 sums (the block's row groups, then 152
-// partials a column by the block's warps) took 2 to 4 us of a launch: mean of a restart cycle of
-// 100 f32 128^3 75.5 -> 71.8 us, i16 101^3 40.2 -> 36.6, bf16 524,288 rows 17.5 -> 14.9, f64 96^3
-// 80.0 -> 78.1.
-__device__ __forceinline__ void dot_finish(const DotArgs& a, const float2* tot, int ncols, long long limit, int* fault)
+// cross-block sum is in FP64 and spread over all SMs: an FP64 instruction occupies GB300's pipe for
+// 20 cycles per SM, so a few columns per block cost little, where 152 partials of every
+// column added by one block took 2 to 4 us of a launch.
+__device__ __forceinline__ void dot_finish(const DotArgs& a, int ncols, long long limit, int* fault)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    float2* part = reinterpret_cast<float2*>(a.part);
-    for (int col = threadIdx.x; col < ncols; col += blockDim.x) part[(long long)blockIdx.x * MAXCOLS + col] = tot[col];
     if (!grid_barrier(a.counter, limit)) {
         if (threadIdx.x == 0) record_fault(nullptr, fault);
         return;
     }
     const int nb = gridDim.x;
     for (int col = blockIdx.x + warp * nb; col < ncols; col += nw * nb) {
-        float S = 0.f, C = 0.f;
+        double s = 0.0;
         for (int t0 = 0; t0 < nb; t0 += 160) {
-            float2 v[5];
+            double v[5];
 #pragma unroll
             for (int u = 0; u < 5; u++) {
                 const int t = t0 + lane + 32 * u;
-                v[u] = t < nb ? __ldcg(part + (long long)t * MAXCOLS + col) : make_float2(0.f, 0.f);
+                v[u] = t < nb ? __ldcg(a.part + (long long)t * MAXCOLS + col) : 0.0;
             }
 #pragma unroll
-            for (int u = 0; u < 5; u++) df_add(S, C, v[u].x, v[u].y);
+            for (int u = 0; u < 5; u++) s = __dadd_rn(s, v[u]);
         }
-        df_warp_sum(S, C);
-        if (lane == 0) a.out[col] = df_to_double(S, C) * a.scales[col];
+        s = warp_sum(s);
+        if (lane == 0) a.out[col] = s * a.scales[col];
     }
 }
 
@@ -264,7 +260,7 @@ __global__ void __launch_bounds__(DOT_THREADS, 1) k_basis_dot_tma(DotArgs a, int
     uint64_t* full = reinterpret_cast<uint64_t*>(tma_smem + (size_t)stages * G::STAGE_DOT);
     uint64_t* empty = full + stages;
     __shared__ float2 red_g[2][TMA_CW][CG];   // per row group sums of the current group (double-buffered)
-    __shared__ float2 red_tot[MAXCOLS];       // the block's column totals
+    __shared__ double red_tot[MAXCOLS];       // the block's column totals
     __shared__ int failed;
     const int ncols = a.ncols_dev ? *a.ncols_dev : a.ncols;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -282,7 +278,7 @@ __global__ void __launch_bounds__(DOT_THREADS, 1) k_basis_dot_tma(DotArgs a, int
         }
         mbar_init_fence();
     }
-    for (int i = threadIdx.x; i < MAXCOLS; i += DOT_THREADS) red_tot[i] = make_float2(0.f, 0.f);
+    for (int i = threadIdx.x; i < MAXCOLS; i += DOT_THREADS) red_tot[i] = 0.0;
     __syncthreads();
 
     if (warp == DOT_CW) {
@@ -330,18 +326,22 @@ __global__ void __launch_bounds__(DOT_THREADS, 1) k_basis_dot_tma(DotArgs a, int
             if ((lane & LOW) == 0) red_g[g & 1][rgp][q0 + col] = make_float2(S[0], C[0]);
             consumers_sync();
             // red_g[g & 1] is rewritten two groups later, after the next barrier
+            // (the row groups added in FP64, a lane each)
             const int tid = warp * 32 + lane;
-            if (tid < nc) {
-                float2 tot = red_g[g & 1][0][tid];
+            if (tid < CG * TMA_CW) {
+                const int c = tid / TMA_CW;
+                const float2 v = c < nc ? red_g[g & 1][tid % TMA_CW][c] : make_float2(0.f, 0.f);
+                double s = df_to_double(v.x, v.y);
 #pragma unroll
-                for (int w = 1; w < TMA_CW; w++) df_add(tot.x, tot.y, red_g[g & 1][w][tid].x, red_g[g & 1][w][tid].y);
-                red_tot[c0 + tid] = tot;
+                for (int o = TMA_CW / 2; o > 0; o >>= 1) s = __dadd_rn(s, __shfl_xor_sync(0xffffffffu, s, o));
+                if (tid % TMA_CW == 0 && c < nc) red_tot[c0 + c] = s;
             }
         }
     }
     __syncthreads();
     if (failed && threadIdx.x == 0) record_fault(nullptr, fault);
-    dot_finish(a, red_tot, ncols, limit, fault);
+    for (int col = threadIdx.x; col < ncols; col += DOT_THREADS) a.part[(long long)blockIdx.x * MAXCOLS + col] = red_tot[col];
+    dot_finish(a, ncols, limit, fault);
 }
 
 // =============================================== w -= V h, u = V^T w in one pass over V
@@ -383,7 +383,7 @@ template <int FMT> struct PassGeom {
     static constexpr int SPAN = 32 * E;                            // rows of a span
     static constexpr int HE = E > 8 ? 8 : E;                       // rows a lane works on at a time
     static constexpr int COEF = PS_MAXC * 24;
-    static constexpr int STATIC = PS_WARPS * 16 * 8 + PS_MAXC * 8 + 128;
+    static constexpr int STATIC = PS_WARPS * 16 * 8 + 128;
     // threads that add one row's sets
     static constexpr __host__ __device__ int lanes(int rs)
     {
@@ -503,7 +503,6 @@ __global__ void __launch_bounds__(PS_THREADS, 1) k_basis_pass(PassArgs a, int sl
                                            PS_GROUPS * G::exch_floats(rs) * 4);      // (c, c, -c, -c)
     float2* cb = reinterpret_cast<float2*>(ca + PS_MAXC);                            // (c low, c low)
     __shared__ float2 red_w[PS_WARPS][16];
-    __shared__ float2 red_tot[PS_MAXC];
     const long long limit = a.d.wait_limit > 0 ? a.d.wait_limit : WAIT_LIMIT_CYCLES;
     long long tb, te;
     block_items(a.d.nrows / rows, tb, te);
@@ -730,12 +729,12 @@ __global__ void __launch_bounds__(PS_THREADS, 1) k_basis_pass(PassArgs a, int sl
     if ((lane & fold_low<16>()) == 0) red_w[warp][q] = make_float2(S[0], C[0]);
     __syncthreads();
     for (int c = threadIdx.x; c < ncols; c += PS_THREADS) {
-        float2 tot = make_float2(0.f, 0.f);
-        for (int w = c % sets; w < PS_WARPS; w += sets) df_add(tot.x, tot.y, red_w[w][c / sets].x, red_w[w][c / sets].y);
-        red_tot[c] = tot;
+        float4 tot = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        for (int w = c % sets; w < PS_WARPS; w += sets) tf_add(tot, red_w[w][c / sets].x, red_w[w][c / sets].y);
+        a.d.part[(long long)blockIdx.x * MAXCOLS + c] = tf_to_double(tot);
     }
-    __syncthreads();
-    dot_finish(a.d, red_tot, ncols, limit, fault);
+    dot_finish(a.d, ncols, limit, fault);
 }
 
 }  // namespace cbg

@@ -1502,7 +1502,7 @@ int cbgmres_create(const cbg_csr* A, int restart, int fmt, const cbg_options* op
     size_t o_h = take(sizeof(double) * ldh), o_u = take(sizeof(double) * ldh);
     size_t o_sc = take(sizeof(double) * ldh);
     size_t o_part = take(sizeof(double) * (size_t)h->gridmax * MAXCOLS);
-    size_t o_pn = take(sizeof(double) * (size_t)h->gridmax * 2);
+    size_t o_pn = take(sizeof(double) * (size_t)h->gridmax * 4);
     size_t o_ps = take(sizeof(double) * (size_t)h->gridmax * 2);
     size_t o_cnt = take(sizeof(unsigned int) * 16);
     // one launch per restart cycle: the default arithmetic and orthogonalisation; profiling
@@ -1950,7 +1950,7 @@ int cbg_basis_axpy(int fmt, int arith, int64_t n, int ncols, const void* V, int6
     Scratch sc(s);
     double* scl = sc.take<double>(ncols);
     double* cf = sc.take<double>(ncols);
-    double* pn = sc.take<double>((size_t)grid * 2);
+    double* pn = sc.take<double>((size_t)grid * 4);
     int rc = sc.alloc();
     if (rc) return rc;
     scl = sc.at(scl); cf = sc.at(cf); pn = sc.at(pn);
