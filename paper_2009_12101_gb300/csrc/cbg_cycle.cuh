@@ -22,8 +22,8 @@
 // SpMV's gather goes to L2.
 //
 // Arithmetic is that of the stepwise kernels: double-float products and sums, the same
-// splits and epilogues; only the order of the sums differs (block partials are combined as
-// double-float pairs).
+// splits and epilogues; only the order of the sums differs, and the columns' sums over blocks are
+// of double-float pairs (see collect).
 //
 // What bounds it: 64^2 f64, restart 100, takes 18 us per step (72 us as separate kernels): 11.5k
 // of 36k cycles in the four barriers (about 1.4 us each: one release, one poll), 6k in the
@@ -62,14 +62,16 @@ struct CycleArgs {
     double* z;
     int lanes;                // SpMV lanes per row (power of two, at most 32)
     int hexp;                 // StoreArgs::hexp
-    float2* part;             // [2][MAXCOLS + 1][CY_MAXG] column partials: h (and omega^2), u
-    float2* norm;             // [2][CY_MAXG] sums of squares, maxima
+    float2* part;             // [2][MAXCOLS][CY_MAXG] column partials: h, u
+    float4* norm;             // [2][CY_MAXG] sums of squares: of w2, omega^2 (triples, see tf_add)
+    float2* wmax;             // [CY_MAXG] maxima
     double* coef;             // [2][2][MAXCOLS] h and u of odd and even steps, for the Givens warp
     unsigned int* counter;    // arrivals; zero when the launch starts
     int* fault;               // set when a wait ran out
     long long limit;          // clock cycles a wait may take
 };
-constexpr size_t CY_PART = (size_t)2 * (MAXCOLS + 1) * CY_MAXG, CY_NORM = (size_t)2 * CY_MAXG, CY_COEF = (size_t)4 * MAXCOLS;
+// their sizes in float2 (8 bytes); norm starts on a 16-byte boundary
+constexpr size_t CY_PART = (size_t)2 * MAXCOLS * CY_MAXG, CY_NORM = (size_t)4 * CY_MAXG, CY_WMAX = CY_MAXG, CY_COEF = (size_t)4 * MAXCOLS;
 
 // shared memory of a block in bytes: planes of w, partial sums of the axpy, per-warp column
 // sums, the resident basis
@@ -88,8 +90,8 @@ template <int FMT> struct CycleGeom {
 struct CycleShared {
     double sR[MAXCOLS + 1], sRo[MAXCOLS + 1], scs[MAXCOLS], ssn[MAXCOLS];   // Givens warp
     double scale[MAXCOLS + 1];
-    float2 cs[MAXCOLS + 1];                    // axpy coefficients (and -omega^2 behind them)
-    float2 wsum[CY_WARPS];                     // per warp sums of squares
+    float2 cs[MAXCOLS];                        // axpy coefficients
+    float4 wsum[CY_WARPS];                     // per warp sums of squares
     float2 wmax[CY_WARPS];                     // per warp maxima
     double hn, inv, omega[2];
     EncParams ep;
@@ -266,8 +268,9 @@ template <int FMT, bool RES> struct Cycle {
                 }
             }
         }
-        df_warp_sum(ssS, ssC);
-        if ((threadIdx.x & 31) == 0) sm.wsum[threadIdx.x >> 5] = make_float2(ssS, ssC);
+        float4 ss = make_float4(ssS, ssC, 0.f, 0.f);
+        tf_warp_sum<true>(ss);
+        if ((threadIdx.x & 31) == 0) sm.wsum[threadIdx.x >> 5] = ss;
     }
 
     // z = P v on the own rows (FP64, as the stepwise kernel)
@@ -289,8 +292,7 @@ template <int FMT, bool RES> struct Cycle {
 
     // The block's partial sums of V^T w over its rows, published as column partials.  The
     // warps are dealt out as wr row splits x wc column groups so that the slowest warp has
-    // the fewest (group, segment) items.  omega: also the warps' sums of squares, as column
-    // ncols.
+    // the fewest (group, segment) items.  omega: also the warps' sums of squares.
     static __device__ void dot(const CycleArgs& a, CycleShared& sm, float2* red, const unsigned char* vs,
                                long long vstride, int R, int ncols, const float* wh, const float* wl, float2* part,
                                bool omega)
@@ -378,32 +380,44 @@ template <int FMT, bool RES> struct Cycle {
             part[c * CY_MAXG + b] = t;
         }
         if (omega && warp == CY_WARPS - 1) {
-            const float2 t = fold_warps(sm.wsum, lane);
-            if (lane == 0) part[ncols * CY_MAXG + b] = t;
+            const float4 t = fold_warps(sm.wsum, lane);
+            if (lane == 0) a.norm[CY_MAXG + b] = t;
         }
     }
 
-    // the sum of the warps' pairs (one warp calls it; all its lanes hold the result)
-    static __device__ float2 fold_warps(const float2* w, int lane)
+    // the sum of the warps' triples (one warp calls it; all its lanes hold the result)
+    static __device__ float4 fold_warps(const float4* w, int lane)
     {
-        float2 t = w[lane & (CY_WARPS - 1)];
+        float4 t = w[lane & (CY_WARPS - 1)];
 #pragma unroll
-        for (int o = CY_WARPS / 2; o > 0; o >>= 1) {
-            const float s2 = __shfl_xor_sync(0xffffffffu, t.x, o), c2 = __shfl_xor_sync(0xffffffffu, t.y, o);
-            df_add(t.x, t.y, s2, c2);
-        }
+        for (int o = CY_WARPS / 2; o > 0; o >>= 1) tf_add(t, tf_shfl_xor(t, o));
         return t;
     }
+    // the sum of the blocks' triples (one warp; its lanes add the blocks lane, lane + 32, ...)
+    static __device__ float4 sum_blocks(const float4* p, int lane)
+    {
+        float4 v[CY_MAXG / 32];                                // all of them in flight at once
+#pragma unroll
+        for (int u = 0; u < CY_MAXG / 32; u++)
+            v[u] = lane + 32 * u < (int)gridDim.x ? __ldcg(p + lane + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int u = 1; u < CY_MAXG / 32; u++) tf_add(v[0], v[u]);
+        tf_warp_sum<true>(v[0]);
+        return v[0];
+    }
 
-    // After the barrier: the sums of all k columns over the blocks (warp w takes the columns
+    // After the barrier: the sums of all columns over the blocks (warp w takes the columns
     // 4 w .. 4 w + 3, then 64 further on; its lanes add the blocks lane, lane + 32, ...) and
-    // from them the axpy's coefficients -scale h in sm.cs; block 0 also keeps h (hout) and
-    // omega^2 (*om, column ncols when k = ncols + 1).
-    static __device__ void collect(const CycleArgs& a, CycleShared& sm, const float2* part, int ncols, int k,
-                                   double* hout, double* om)
+    // from them the axpy's coefficients -scale h in sm.cs; block 0 also keeps h (hout).  These sums
+    // are double-float: the second projection takes in what the first one missed, and h is recorded
+    // as the pair that the subtraction uses, so that it is as close to 64 bits as from the
+    // stepwise kernels, or closer (29,791 rows f32, rms of ||h||: 1.4e-16, stepwise 1.0e-15; triples
+    // of floats gave 5e-16, a tenth slower).  The norms have no second pass, and double-float sums
+    // doubled their error.
+    static __device__ void collect(const CycleArgs& a, CycleShared& sm, const float2* part, int ncols, double* hout)
     {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nb = gridDim.x;
-        for (int c0 = 4 * warp; c0 < k; c0 += 4 * CY_WARPS) {
+        for (int c0 = 4 * warp; c0 < ncols; c0 += 4 * CY_WARPS) {
             float S[4], C[4];
 #pragma unroll
             for (int q = 0; q < 4; q++) S[q] = C[q] = 0.f;
@@ -412,7 +426,7 @@ template <int FMT, bool RES> struct Cycle {
             for (int u = 0; u < CY_MAXG / 32; u++)
 #pragma unroll
                 for (int q = 0; q < 4; q++)
-                    v[u][q] = lane + 32 * u < nb && c0 + q < k ? __ldcg(part + (c0 + q) * CY_MAXG + lane + 32 * u)
+                    v[u][q] = lane + 32 * u < nb && c0 + q < ncols ? __ldcg(part + (c0 + q) * CY_MAXG + lane + 32 * u)
                                                                : make_float2(0.f, 0.f);
 #pragma unroll
             for (int u = 0; u < CY_MAXG / 32; u++) {
@@ -421,7 +435,7 @@ template <int FMT, bool RES> struct Cycle {
                 for (int q = 0; q < 4; q++) df_add(S[q], C[q], v[u][q].x, v[u][q].y);
             }
             const int c = c0 + df_warp_fold<4>(S, C, lane);
-            if ((lane & 7) == 0 && c < k) {
+            if ((lane & 7) == 0 && c < ncols) {
                 float h, l;                                    // -(the sum), renormalised
                 two_sum(-S[0], -C[0], h, l);
                 sm.cs[c] = make_float2(h, l);
@@ -432,21 +446,17 @@ template <int FMT, bool RES> struct Cycle {
         // there in as few warps as there are columns: an FP64 instruction occupies GB300's
         // narrow pipe for a whole warp however few lanes take part
         if (blockIdx.x == 0 || SCALED) {
-            for (int c = threadIdx.x; c < k; c += CY_CT) {
+            for (int c = threadIdx.x; c < ncols; c += CY_CT) {
                 const float2 v = sm.cs[c];
                 double h = -df_to_double(v.x, v.y);
-                if (c < ncols) {
-                    if constexpr (SCALED) {
-                        const double sc = sm.scale[c];
-                        h = __dmul_rn(h, sc);
-                        float hi, lo;
-                        split_f64(-__dmul_rn(sc, h), hi, lo);
-                        sm.cs[c] = make_float2(hi, lo);
-                    }
-                    if (blockIdx.x == 0) hout[c] = h;
-                } else if (blockIdx.x == 0) {
-                    *om = h;
+                if constexpr (SCALED) {
+                    const double sc = sm.scale[c];
+                    h = __dmul_rn(h, sc);
+                    float hi, lo;
+                    split_f64(-__dmul_rn(sc, h), hi, lo);
+                    sm.cs[c] = make_float2(hi, lo);
                 }
+                if (blockIdx.x == 0) hout[c] = h;
             }
             cy_sync();
         }
@@ -561,10 +571,11 @@ template <int FMT, bool RES> struct Cycle {
             }
         }
         if constexpr (NORMS) {
-            df_warp_sum(ssS, ssC);
+            float4 ss = make_float4(ssS, ssC, 0.f, 0.f);
+            tf_warp_sum<true>(ss);
             fold_max(mx);
             if ((threadIdx.x & 31) == 0) {
-                sm.wsum[threadIdx.x >> 5] = make_float2(ssS, ssC);
+                sm.wsum[threadIdx.x >> 5] = ss;
                 sm.wmax[threadIdx.x >> 5] = mx;
             }
         }
@@ -585,37 +596,37 @@ template <int FMT, bool RES> struct Cycle {
     {
         if (threadIdx.x < 32) {
             const int lane = threadIdx.x;
-            const float2 s = fold_warps(sm.wsum, lane);
+            const float4 s = fold_warps(sm.wsum, lane);
             float2 m = sm.wmax[lane & (CY_WARPS - 1)];
             fold_max(m);
             if (lane == 0) {
                 a.norm[blockIdx.x] = s;
-                a.norm[CY_MAXG + blockIdx.x] = m;
+                a.wmax[blockIdx.x] = m;
             }
         }
     }
-    // after the barrier: those of all blocks, and what the encoding of column col needs
-    static __device__ void collect_norms(const CycleArgs& a, CycleShared& sm, int col)
+    // after the barrier: those of all blocks, and what the encoding of column col needs; block 0
+    // also sums omega^2 (*om), which only the Givens update reads
+    static __device__ void collect_norms(const CycleArgs& a, CycleShared& sm, int col, double* om)
     {
+        if (blockIdx.x == 0 && threadIdx.x >> 5 == 1) {
+            const float4 s = sum_blocks(a.norm + CY_MAXG, threadIdx.x & 31);
+            if (threadIdx.x == 32) *om = tf_to_double<true>(s);
+        }
         if (threadIdx.x < 32) {
             const int lane = threadIdx.x, nb = gridDim.x;
-            float2 v[CY_MAXG / 32], w[CY_MAXG / 32];
+            float2 w[CY_MAXG / 32];
 #pragma unroll
-            for (int u = 0; u < CY_MAXG / 32; u++) {
-                const bool in = lane + 32 * u < nb;
-                v[u] = in ? __ldcg(a.norm + lane + 32 * u) : make_float2(0.f, 0.f);
-                w[u] = in ? __ldcg(a.norm + CY_MAXG + lane + 32 * u) : make_float2(0.f, 0.f);
-            }
-            float2 s = v[0], m = w[0];
+            for (int u = 0; u < CY_MAXG / 32; u++)
+                w[u] = lane + 32 * u < nb ? __ldcg(a.wmax + lane + 32 * u) : make_float2(0.f, 0.f);
+            const float4 s = sum_blocks(a.norm, lane);
+            float2 m = w[0];
 #pragma unroll
-            for (int u = 1; u < CY_MAXG / 32; u++) {
-                df_add(s.x, s.y, v[u].x, v[u].y);
+            for (int u = 1; u < CY_MAXG / 32; u++)
                 if (!(w[u].x < m.x || (w[u].x == m.x && w[u].y <= m.y))) m = w[u];
-            }
-            df_warp_sum(s.x, s.y);
             fold_max(m);
             if (lane == 0) {
-                const double hn = sqrt(df_to_double(s.x, s.y)), inv = 1.0 / hn;
+                const double hn = sqrt(tf_to_double<true>(s)), inv = 1.0 / hn;
                 sm.hn = hn;
                 sm.inv = inv;
                 sm.ep = enc_params(FMT, __dmul_rn(df_to_double(m.x, m.y), inv));
@@ -660,7 +671,7 @@ template <int FMT, bool RES> struct Cycle {
         unsigned char* res = reinterpret_cast<unsigned char*>(red + CY_WARPS * a.mcols);
         const unsigned char* vs = RES ? res : a.V + r0 * BS;          // own rows of column 0
         const long long vstride = RES ? (long long)a.rows * BS : a.ldb;
-        float2* part2 = a.part + (MAXCOLS + 1) * CY_MAXG;
+        float2* part2 = a.part + MAXCOLS * CY_MAXG;
         unsigned epoch = 0;
         volatile int* fail = &sm.fail;
         if (t == 0) sm.scale[0] = a.d.scales[0];
@@ -690,20 +701,20 @@ template <int FMT, bool RES> struct Cycle {
             dot(a, sm, red, vs, vstride, R, ncols, wh, wl, a.part, true);
             cy_grid_sync(a, sm, epoch);
             if (*fail) break;
-            collect(a, sm, a.part, ncols, ncols + 1, hj, &sm.omega[j & 1]);
+            collect(a, sm, a.part, ncols, hj);
             // w1 = w - V h ; u = V^T w1
             axpy<false>(a, sm, vs, vstride, r0, R, ncols, wh, wl, split);
             dot(a, sm, red, vs, vstride, R, ncols, wh, wl, part2, false);
             if (b == 0 && j > 0) cy_take(3);                          // the Givens update of step j - 1
             cy_grid_sync(a, sm, epoch);
             if (*fail || (j > 0 && *(volatile int*)&a.d.st->active == 0)) break;
-            collect(a, sm, part2, ncols, ncols, hj + MAXCOLS, nullptr);
+            collect(a, sm, part2, ncols, hj + MAXCOLS);
             // w2 = w1 - V u, its norms
             axpy<true>(a, sm, vs, vstride, r0, R, ncols, wh, wl, split);
             put_norms(a, sm);
             cy_grid_sync(a, sm, epoch);
             if (*fail) break;
-            collect_norms(a, sm, ncols);
+            collect_norms(a, sm, ncols, &sm.omega[j & 1]);
             if (b == 0) {
                 if (t == 0) a.d.scales[ncols] = sm.ep.scale;
                 cy_post(2);                                           // column j to the Givens warp

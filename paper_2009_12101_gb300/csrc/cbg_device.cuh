@@ -515,16 +515,6 @@ __device__ __forceinline__ double warp_max(double v)
     return v;
 }
 
-// (S, C) summed over the warp in double-float (every lane holds the result)
-__device__ __forceinline__ void df_warp_sum(float& S, float& C)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float s2 = __shfl_xor_sync(0xFFFFFFFFu, S, o), c2 = __shfl_xor_sync(0xFFFFFFFFu, C, o);
-        df_add(S, C, s2, c2);
-    }
-}
-
 // Sums of FP32 pairs across threads, warps and blocks without loss against FP64 additions and
 // without the FP64 pipe: three floats x + y + z.  x and y take the sum and its rounding errors by
 // two_sum, z what remains of those, so an addition loses about 2^-70 of the sum (FP64: 2^-53; an
@@ -539,9 +529,11 @@ __device__ __forceinline__ void tf_add(float4& a, float h, float l, float z = 0.
     a.z = __fadd_rn(__fadd_rn(a.z, z), __fadd_rn(f, g));
 }
 __device__ __forceinline__ void tf_add(float4& a, const float4& b) { tf_add(a, b.x, b.y, b.z); }
-__device__ __forceinline__ double tf_to_double(const float4& a)
+// HOT, here and below: for code that runs many times in a launch (the other form is the shorter one)
+template <bool HOT = false> __device__ __forceinline__ double tf_to_double(const float4& a)
 {
-    return __dadd_rn((double)a.x, __dadd_rn((double)a.y, (double)a.z));
+    if constexpr (HOT) return __dadd_rn(f32_to_f64_exact(a.x), __dadd_rn(f32_to_f64_exact(a.y), f32_to_f64_exact(a.z)));
+    else return __dadd_rn((double)a.x, __dadd_rn((double)a.y, (double)a.z));
 }
 __device__ __forceinline__ float4 tf_shfl_xor(const float4& a, int o)
 {
@@ -551,10 +543,15 @@ __device__ __forceinline__ float4 tf_shfl_xor(const float4& a, int o)
 // (every lane holds the result).  Loops, here and in what uses it: a kernel's tail runs once, and
 // instructions that are fetched for a single use cost more than those that run (written out, the
 // tails of the axpy and of the one-pass kernel took 1 to 3 us longer).
-__device__ __forceinline__ void tf_warp_sum(float4& a)
+template <bool HOT = false> __device__ __forceinline__ void tf_warp_sum(float4& a)
 {
+    if constexpr (HOT) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) tf_add(a, tf_shfl_xor(a, o));
+    } else {
 #pragma unroll 1
-    for (int o = 16; o > 0; o >>= 1) tf_add(a, tf_shfl_xor(a, o));
+        for (int o = 16; o > 0; o >>= 1) tf_add(a, tf_shfl_xor(a, o));
+    }
 }
 
 // The block's sum of the threads' a; valid in warp 0.  red: shared, one entry per warp.  All threads

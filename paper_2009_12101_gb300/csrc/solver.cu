@@ -810,8 +810,9 @@ void enqueue_cycle(cbg_handle* h)
     a.lanes = h->cycle_lanes;
     a.hexp = -h->pexp;
     a.part = h->cycle_part;
-    a.norm = a.part + CY_PART;
-    a.coef = reinterpret_cast<double*>(a.norm + CY_NORM);
+    a.norm = reinterpret_cast<float4*>(a.part + CY_PART);
+    a.wmax = a.part + CY_PART + CY_NORM;
+    a.coef = reinterpret_cast<double*>(a.wmax + CY_WMAX);
     a.counter = h->d.counters + CNT_CYCLE;
     a.fault = &h->d.st->fault;
     a.limit = WAIT_LIMIT_CYCLES;
@@ -1509,7 +1510,7 @@ int cbgmres_create(const cbg_csr* A, int restart, int fmt, const cbg_options* op
     // times the kernels of a step, so it keeps them apart
     const bool single = o.arith == CBG_ARITH_DF32 && o.ortho == CBG_ORTHO_CGS && o.reorth == CBG_REORTH_ALWAYS &&
                         h->valdf && !o.profile && cycle_worthwhile(n, nnz, restart, fmt);
-    size_t o_cyc = single ? take(sizeof(float2) * (CY_PART + CY_NORM + CY_COEF)) : 0;
+    size_t o_cyc = single ? take(sizeof(float2) * (CY_PART + CY_NORM + CY_WMAX + CY_COEF)) : 0;
     unsigned char* blk = nullptr;
     TRY(dalloc(&blk, off));
     h->state_block = blk;

@@ -66,3 +66,10 @@ def test_norm_of_the_new_vector_stepwise(fmt, n):
     torch, cb = need_gpu()
     err = _new_vector_norms(cb, torch, fmt, n, profile=True)
     assert np.sqrt(np.mean(np.square(err))) <= 4e-16, err
+
+
+@pytest.mark.parametrize("fmt", ["f32", "e4m3"])
+def test_norm_of_the_new_vector_single_launch(fmt):
+    torch, cb = need_gpu()
+    err = _new_vector_norms(cb, torch, fmt, 262144, profile=False)
+    assert np.sqrt(np.mean(np.square(err))) <= 4e-16, err
