@@ -638,8 +638,8 @@ template <int FMT> struct BatchedSolver {
         __syncthreads();
     }
 
-    // w -= V coef over own rows; with NORMS, also the block's sum of squares (double-float,
-    // into sm->red[0]) and, for the formats whose scale needs it, the maximum of |w| (into
+    // w -= V coef over own rows; with NORMS, also the block's sum of squares (triples of floats,
+    // tf_add, into sm->red[0]) and, for the formats whose scale needs it, the maximum of |w| (into
     // sm->red[1]).  Blocks with fewer row chunks than threads split the columns over the
     // lanes of a warp; the column loads are software-pipelined.
     template <bool NORMS>
@@ -647,7 +647,8 @@ template <int FMT> struct BatchedSolver {
                                 const double* coef)
     {
         __shared__ float2 cdf[BT_MAXM + 1];
-        __shared__ float2 wsum[NW], wmax[NW];
+        __shared__ float4 wsum[NW];
+        __shared__ float2 wmax[NW];
         for (int k = threadIdx.x; k < ncols; k += BT_THREADS) {
             float hi, lo;
             split_f64(-coef[k] * sm->scale[k], hi, lo);
@@ -663,7 +664,7 @@ template <int FMT> struct BatchedSolver {
         int lk = 0;                                            // 2^lk column splits
         while (lk < 3 && (nch << (lk + 1)) <= BT_THREADS) lk++;
         const int ks = 1 << lk, cpw = 32 >> lk, mk = lane >> (5 - lk), mch = lane & (cpw - 1);
-        float ssS = 0.f, ssC = 0.f;
+        float4 ss = make_float4(0.f, 0.f, 0.f, 0.f);
         float2 mx = make_float2(0.f, 0.f);
         for (int base = warp * cpw; base < nch; base += NW * cpw) {
             const int ch = base + mch;
@@ -724,13 +725,12 @@ template <int FMT> struct BatchedSolver {
                     sm->w[r] = h;
                     wl[r] = l;
                     if constexpr (NORMS) {
-                        const float p = __fmul_rn(h, h);       // h^2 + 2 h l
-                        float q = __fmaf_rn(h, h, -p);
-                        q = __fmaf_rn(__fadd_rn(h, h), l, q);
-                        float t, te;
-                        two_sum(ssS, p, t, te);
-                        ssC = __fadd_rn(ssC, __fadd_rn(te, q));
-                        ssS = t;
+                        // h^2 = p + q and 2 h l = t + u exactly, l^2
+                        const float p = __fmul_rn(h, h), q = __fmaf_rn(h, h, -p);
+                        const float h2 = __fadd_rn(h, h), t = __fmul_rn(h2, l), u = __fmaf_rn(h2, l, -t);
+                        float y, z;
+                        two_sum(t, q, y, z);
+                        tf_add(ss, p, y, __fadd_rn(z, __fmaf_rn(l, l, u)));
                         if constexpr (SCALED) {
                             const float ah = fabsf(h), al = h < 0.f ? -l : l;
                             if (!(ah < mx.x || (ah == mx.x && al <= mx.y))) mx = make_float2(ah, al);
@@ -742,25 +742,25 @@ template <int FMT> struct BatchedSolver {
         if constexpr (NORMS) {
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
-                const float oS = __shfl_xor_sync(0xffffffffu, ssS, o), oC = __shfl_xor_sync(0xffffffffu, ssC, o);
-                df_add(ssS, ssC, oS, oC);
+                tf_add(ss, tf_shfl_xor(ss, o));
                 if constexpr (SCALED) {
                     const float h2 = __shfl_xor_sync(0xffffffffu, mx.x, o), l2 = __shfl_xor_sync(0xffffffffu, mx.y, o);
                     if (!(h2 < mx.x || (h2 == mx.x && l2 <= mx.y))) mx = make_float2(h2, l2);
                 }
             }
             if (lane == 0) {
-                wsum[warp] = make_float2(ssS, ssC);
+                wsum[warp] = ss;
                 wmax[warp] = mx;
             }
             __syncthreads();
             if (threadIdx.x == 0) {
-                float2 t = wsum[0], m = wmax[0];
+                float4 t = wsum[0];
+                float2 m = wmax[0];
                 for (int w = 1; w < NW; w++) {
-                    df_add(t.x, t.y, wsum[w].x, wsum[w].y);
+                    tf_add(t, wsum[w]);
                     if (!(wmax[w].x < m.x || (wmax[w].x == m.x && wmax[w].y <= m.y))) m = wmax[w];
                 }
-                sm->red[0] = df_to_double(t.x, t.y);
+                sm->red[0] = tf_to_double<true>(t);
                 sm->red[1] = df_to_double(m.x, m.y);
             }
         }
