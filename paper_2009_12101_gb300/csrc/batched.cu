@@ -111,15 +111,16 @@ struct cbg_batch {
 
 namespace {
 
-// rows of w one block holds: a cluster share of the largest cooperative system, or a whole
-// small system (and the 16-entry tail the chunked loops read)
+// rows of w one block holds: a cluster share of the largest cooperative system (whole chunks of
+// 32 rows), or a whole small system; a multiple of 16, the most that the loops over 16-byte
+// chunks of codes read past the rows
 long long block_rows(const cbg_batch* bt, const Schedule& sc)
 {
     long long rows_cluster = sc.cluster > 1 ? ((bt->max_n + sc.cluster - 1) / sc.cluster + 31) / 32 * 32 : 0;
     long long rows_small = 0;
     for (const auto& s : bt->sys)
         if (sc.cluster == 1 || s.n < sc.split_rows) rows_small = std::max<long long>(rows_small, s.n);
-    return (std::max(rows_cluster, rows_small) + 31) / 32 * 32 + 16;
+    return (std::max(rows_cluster, rows_small) + 15) / 16 * 16;
 }
 
 size_t smem_bytes(const cbg_batch* bt, const Schedule& sc)

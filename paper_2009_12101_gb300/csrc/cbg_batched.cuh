@@ -88,7 +88,8 @@ struct BtSmem {
     double h[BT_MAXM + 1], u[BT_MAXM + 1], scale[BT_MAXM + 1];
     double red[BT_MAXM + 4];           // this block's partial sums (read by the cluster)
     double tot[BT_MAXM + 4];           // team totals
-    double wred[BT_THREADS / 32][BT_MAXM + 4];   // (the dot: row splits' sums as float2)
+    alignas(16) double wred[BT_THREADS / 32][BT_MAXM + 4];   // (the dot: row splits' sums as float2; the
+                                                             // axpy: the warps' norms)
     double inv, omega;                 // of the current step (formed by one thread: an FP64 instruction
     EncParams ep;                      // occupies the narrow pipe for a whole warp)
     int sys_idx;
@@ -647,8 +648,8 @@ template <int FMT> struct BatchedSolver {
                                 const double* coef)
     {
         __shared__ float2 cdf[BT_MAXM + 1];
-        __shared__ float4 wsum[NW];
-        __shared__ float2 wmax[NW];
+        float4* wsum = reinterpret_cast<float4*>(&sm->wred[0][0]);     // (shared memory bounds the systems' size)
+        float2* wmax = reinterpret_cast<float2*>(wsum + NW);
         for (int k = threadIdx.x; k < ncols; k += BT_THREADS) {
             float hi, lo;
             split_f64(-coef[k] * sm->scale[k], hi, lo);
@@ -852,8 +853,8 @@ template <int FMT> struct BatchedSolver {
         const int r1 = min(s.n, r0 + chunk);
         const int nloc = r1 - r0;
         float* wl = sm->w + a.max_rows_block;
-        // zero the w rows (and the 16-entry tail read by the chunked loops)
-        for (int i = threadIdx.x; i < nloc + 16; i += BT_THREADS) sm->w[i] = wl[i] = 0.f;
+        // zero the w rows, and those up to the next 16, which the chunked loops read
+        for (int i = threadIdx.x; i < (nloc + 15) / 16 * 16; i += BT_THREADS) sm->w[i] = wl[i] = 0.f;
         double* x = a.io[1] + s.vec_off;
         const double* dinv = a.dinv ? a.dinv + s.vec_off : nullptr;
 
