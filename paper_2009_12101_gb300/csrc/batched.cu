@@ -185,12 +185,48 @@ __global__ void k_batch_sell(const BatchSys* sys, const int* csys, long long nch
     }
 }
 
+void free_sell(cbg_batch* bt)
+{
+    cudaFree(bt->d_soff); cudaFree(bt->d_scol); cudaFree(bt->d_sval); cudaFree(bt->d_sval64);
+    bt->d_soff = nullptr;
+    bt->d_scol = nullptr;
+    bt->d_sval = nullptr;
+    bt->d_sval64 = nullptr;
+}
+
+// The sliced-ELL copy on the device (csys: the chunks' systems, soff: their offsets).  Not enough
+// memory for it is no error.
+int build_sell(cbg_batch* bt, const std::vector<int>& csys, const std::vector<long long>& soff)
+{
+    int* d_csys = nullptr;
+    cudaError_t e = cudaMalloc((void**)&d_csys, csys.size() * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&bt->d_soff, soff.size() * sizeof(long long));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&bt->d_scol, bt->sell_entries * sizeof(int));
+    if (e == cudaSuccess)
+        e = cudaMalloc(bt->fmt == CBG_F64 ? (void**)&bt->d_sval64 : (void**)&bt->d_sval, bt->sell_entries * sizeof(double));
+    if (e == cudaSuccess) e = cudaMemcpy(d_csys, csys.data(), csys.size() * sizeof(int), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(bt->d_soff, soff.data(), soff.size() * sizeof(long long), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        const long long nch = (long long)csys.size();
+        k_batch_sell<<<(int)std::min<long long>((nch * 32 + 255) / 256, 4096), 256>>>(
+            bt->d_sys, d_csys, nch, bt->d_rowptr, bt->d_col, bt->d_valpdf, bt->total_nnz,
+            bt->d_valp ? bt->d_valp : bt->d_val, bt->d_soff, bt->sell_entries, bt->d_scol, bt->d_sval, bt->d_sval64);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(0);
+    }
+    cudaFree(d_csys);
+    if (e == cudaSuccess) return CBG_OK;
+    free_sell(bt);
+    cudaGetLastError();                                  // (a failed allocation is not the next call's error)
+    return e == cudaErrorMemoryAllocation ? CBG_OK : CBG_ERR_CUDA;
+}
+
 void free_batch(cbg_batch* bt)
 {
     if (!bt) return;
     cudaFree(bt->d_sys); cudaFree(bt->d_order); cudaFree(bt->d_rowptr); cudaFree(bt->d_col);
     cudaFree(bt->d_val); cudaFree(bt->d_valp); cudaFree(bt->d_dinv); cudaFree(bt->d_valpdf);
-    cudaFree(bt->d_soff); cudaFree(bt->d_scol); cudaFree(bt->d_sval); cudaFree(bt->d_sval64);
+    free_sell(bt);
     cudaFree(bt->d_V); cudaFree(bt->d_out);
     cudaFree(bt->d_queue); cudaFree(bt->d_io);
     if (bt->h_io) cudaFreeHost(bt->h_io);
@@ -527,23 +563,6 @@ int cbgmres_create_batched(int nsys, const cbg_csr* As, int restart, int fmt, co
     soff.push_back(bt->sell_entries);
     const bool sell = !rc && sell_fmt && bt->sell_entries <= bt->total_nnz + bt->total_nnz / 4;
     rc = rc ? rc : up((void**)&bt->d_sys, bt->sys.data(), bt->sys.size() * sizeof(BatchSys));
-    if (!rc && sell) {
-        int* d_csys = nullptr;
-        rc = up((void**)&d_csys, csys.data(), csys.size() * sizeof(int));
-        rc = rc ? rc : up((void**)&bt->d_soff, soff.data(), soff.size() * sizeof(long long));
-        if (!rc && (cudaMalloc((void**)&bt->d_scol, bt->sell_entries * sizeof(int)) != cudaSuccess ||
-                    cudaMalloc(fmt == CBG_F64 ? (void**)&bt->d_sval64 : (void**)&bt->d_sval,
-                               bt->sell_entries * sizeof(double)) != cudaSuccess))
-            rc = CBG_ERR_OOM;
-        if (!rc) {
-            const long long nch = (long long)csys.size();
-            k_batch_sell<<<(int)std::min<long long>((nch * 32 + 255) / 256, 4096), 256>>>(
-                bt->d_sys, d_csys, nch, bt->d_rowptr, bt->d_col, bt->d_valpdf, bt->total_nnz,
-                bt->d_valp ? bt->d_valp : bt->d_val, bt->d_soff, bt->sell_entries, bt->d_scol, bt->d_sval, bt->d_sval64);
-            if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(0) != cudaSuccess) rc = CBG_ERR_CUDA;
-        }
-        cudaFree(d_csys);
-    }
     if (!rc && cudaMalloc((void**)&bt->d_V, std::max<long long>(v_off, 256)) != cudaSuccess) rc = CBG_ERR_OOM;
     if (!rc && cudaMemset(bt->d_V, 0, std::max<long long>(v_off, 256)) != cudaSuccess) rc = CBG_ERR_CUDA;
     if (!rc && cudaMalloc((void**)&bt->d_out, nsys * sizeof(BatchOut)) != cudaSuccess) rc = CBG_ERR_OOM;
@@ -552,6 +571,8 @@ int cbgmres_create_batched(int nsys, const cbg_csr* As, int restart, int fmt, co
     if (!rc && cudaHostAlloc((void**)&bt->h_io, 2 * sizeof(double*), cudaHostAllocDefault) != cudaSuccess) rc = CBG_ERR_OOM;
     if (!rc && (cudaEventCreate(&bt->e0) != cudaSuccess || cudaEventCreate(&bt->e1) != cudaSuccess)) rc = CBG_ERR_CUDA;
     if (!rc && cudaStreamCreateWithFlags(&bt->capture, cudaStreamNonBlocking) != cudaSuccess) rc = CBG_ERR_CUDA;
+    // last, because the solver does without it (the CSR planes) when the memory is short
+    if (!rc && sell) rc = build_sell(bt, csys, soff);
     if (rc) {
         free_batch(bt);
         return rc;
