@@ -732,7 +732,7 @@ double store_bytes(const cbg_handle* h) { return (double)h->n * (8.0 + (double)f
 // ------------------------------------------------------------------ launches per step
 void plan_cycle(cbg_handle* h);
 
-// Basis format of the following cycles: code stride and the format-dependent grids.
+// Basis format: code stride and the format-dependent grids.
 void set_format(cbg_handle* h, int fmt)
 {
     const Ops& op = ops_for(fmt);
@@ -743,6 +743,17 @@ void set_format(cbg_handle* h, int fmt)
     const long long axpy_blocks = h->ld / ((long long)THREADS * (16 / fmt_bytes(fmt)));
     h->grid_axpy = std::max(1, (int)std::min<long long>(axpy_blocks, (long long)sms * std::max(1, op.occ_axpy())));
     plan_cycle(h);
+}
+
+// set_format between cycles.  The columns move with their stride: what is now their rows n .. ld-1
+// may hold codes of the old format, and every kernel reads whole tiles.
+int change_format(cbg_handle* h, int fmt)
+{
+    set_format(h, fmt);
+    const long long bs = fmt_bytes(fmt);
+    if (h->ld > h->n)
+        CBG_CUDA(cudaMemset2DAsync(h->V + h->n * bs, h->ldb, 0, (h->ld - h->n) * bs, h->m + 1, h->stream));
+    return CBG_OK;
 }
 
 // Whether a restart cycle runs as one launch (cbg_cycle.cuh), and how.  Measured against the
@@ -1148,7 +1159,10 @@ int run_solve(cbg_handle* h, const double* b, double* x, double tol, long long m
 {
     if (!h || !b || !x || !(tol >= 0.0) || maxit < 0) return CBG_ERR_ARG;
     cudaStream_t s = h->stream;
-    if (h->fmt != h->fmt0) set_format(h, h->fmt0);   // every solve starts in the handle's format
+    if (h->fmt != h->fmt0) {                         // every solve starts in the handle's format
+        const int rf = change_format(h, h->fmt0);
+        if (rf) return rf;
+    }
     long long promotions = 0;
     CBG_CUDA(cudaEventRecord(h->ev0, s));
     // ||b|| and finiteness of b and x0
@@ -1218,7 +1232,8 @@ int run_solve(cbg_handle* h, const double* b, double* x, double tol, long long m
             if (h->opt.adapt && cycles > 0 && hs.beta > h->opt.adapt_gap * hs.est) {
                 const int nf = promote_format(h->fmt);
                 if (nf >= 0) {
-                    set_format(h, nf);
+                    rc = change_format(h, nf);
+                    if (rc) return rc;
                     promotions++;
                 }
             }
