@@ -2,6 +2,7 @@
 #pragma once
 #include <algorithm>
 
+#include "cbg_context.h"
 #include "cbg_launch.h"
 
 namespace cbg {
@@ -37,16 +38,16 @@ void Launcher<FMT>::axpy(int arith, int epi, int grid, cudaStream_t s, const Axp
 }
 
 // Ring stages of the pipelined dot: the opt-in shared memory left by the kernel's static
-// shared memory (queried once per process), and the matching opt-in attribute.
+// shared memory (queried once per context), and the matching opt-in attribute.
 struct TmaPlan {
     int stages = 0;
     size_t smem = 0;
 };
-template <int FMT> static const TmaPlan& tma_plan()
+template <int FMT> static TmaPlan tma_plan()
 {
-    static const TmaPlan plan = [] {
+    static PerContext<TmaPlan> plan;
+    return plan.get([](TmaPlan& p) {
         using G = TmaGeom<FMT>;
-        TmaPlan p;
         cudaFuncAttributes fa{};
         const int static_bytes =
             cudaFuncGetAttributes(&fa, k_basis_dot_tma<FMT>) == cudaSuccess ? (int)fa.sharedSizeBytes : TMA_SMEM_OPTIN;
@@ -54,9 +55,8 @@ template <int FMT> static const TmaPlan& tma_plan()
         p.smem = tma_smem_bytes(p.stages, G::STAGE_DOT);
         if (p.stages >= 2)
             cudaFuncSetAttribute(k_basis_dot_tma<FMT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
-        return p;
-    }();
-    return plan;
+        return true;
+    });
 }
 
 template <int FMT> bool Launcher<FMT>::tma_fits() { return tma_plan<FMT>().stages >= 2; }
@@ -64,7 +64,7 @@ template <int FMT> bool Launcher<FMT>::tma_fits() { return tma_plan<FMT>().stage
 template <int FMT> void Launcher<FMT>::dot_tma(int grid, cudaStream_t s, const DotArgs& a, int* fault)
 {
     // cooperative: the kernel's blocks meet at a grid barrier before the cross-block sum
-    const TmaPlan& p = tma_plan<FMT>();
+    const TmaPlan p = tma_plan<FMT>();
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(DOT_THREADS);
@@ -80,16 +80,16 @@ template <int FMT> void Launcher<FMT>::dot_tma(int grid, cudaStream_t s, const D
 
 template <int FMT, int RS> static bool pass_kernel_fits()
 {
-    static const bool ok = [] {
+    static PerContext<bool> ok;
+    return ok.get([](bool& good) {
         cudaFuncAttributes fa{};
-        const bool good = cudaFuncGetAttributes(&fa, k_basis_pass<FMT, RS>) == cudaSuccess &&
+        good = cudaFuncGetAttributes(&fa, k_basis_pass<FMT, RS>) == cudaSuccess &&
                           (int)fa.sharedSizeBytes <= PassGeom<FMT>::STATIC &&
                           cudaFuncSetAttribute(k_basis_pass<FMT, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                TMA_SMEM_OPTIN - PassGeom<FMT>::STATIC) == cudaSuccess;
         if (!good) cudaGetLastError();
-        return good;
-    }();
-    return ok;
+        return true;
+    });
 }
 
 template <int FMT> bool Launcher<FMT>::pass_fits(int ncols)
@@ -179,20 +179,21 @@ template <int FMT> int Launcher<FMT>::occupancy_spmv()
 
 namespace cbg {
 
-// dynamic shared memory a block of the cycle kernel may have (opted in once per process)
+// dynamic shared memory a block of the cycle kernel may have (opted in once per context)
 template <int FMT, bool RES> static bool cycle_kernel_fits(size_t smem)
 {
-    static const size_t room = [] {
+    static PerContext<size_t> room;
+    return smem <= room.get([](size_t& r) {
         cudaFuncAttributes fa{};
         if (cudaFuncGetAttributes(&fa, k_cycle<FMT, RES>) != cudaSuccess ||
             cudaFuncSetAttribute(k_cycle<FMT, RES>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  TMA_SMEM_OPTIN - (int)fa.sharedSizeBytes) != cudaSuccess) {
             cudaGetLastError();
-            return (size_t)0;
+            return true;                                // (r = 0)
         }
-        return (size_t)TMA_SMEM_OPTIN - fa.sharedSizeBytes;
-    }();
-    return smem <= room;
+        r = (size_t)TMA_SMEM_OPTIN - fa.sharedSizeBytes;
+        return true;
+    });
 }
 
 template <int FMT, bool RES> static void cycle_kernel_run(int grid, size_t smem, cudaStream_t s, const CycleArgs& a)

@@ -33,6 +33,7 @@
 
 #include <algorithm>
 
+#include "cbg_context.h"
 #include "cbg_device.cuh"
 #include "cbg_mlp.h"
 #include "cbg_tc.cuh"
@@ -535,19 +536,25 @@ int mlp_tc_grid(long long n)
 
 cudaError_t mlp_tc_launch(int mode, int grid, cudaStream_t s, const MlpArgs& a)
 {
-    static bool attr[3] = {false, false, false};
+    static PerContext<cudaError_t> attr[3];
+    auto opt_in = [&](int k, auto kernel) {
+        return attr[k].get([&](cudaError_t& r) {
+            r = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM);
+            return r == cudaSuccess;
+        });
+    };
     cudaError_t e = cudaSuccess;
     switch (mode) {
     case MLP_FWD:
-        if (!attr[0]) { e = cudaFuncSetAttribute(k_mlp_tc<MLP_FWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM); attr[0] = e == cudaSuccess; }
+        e = opt_in(0, k_mlp_tc<MLP_FWD>);
         if (e == cudaSuccess) k_mlp_tc<MLP_FWD><<<grid, MT, MLP_SMEM, s>>>(a);
         break;
     case MLP_BWD:
-        if (!attr[1]) { e = cudaFuncSetAttribute(k_mlp_tc<MLP_BWD>, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM); attr[1] = e == cudaSuccess; }
+        e = opt_in(1, k_mlp_tc<MLP_BWD>);
         if (e == cudaSuccess) k_mlp_tc<MLP_BWD><<<grid, MT, MLP_SMEM, s>>>(a);
         break;
     default:
-        if (!attr[2]) { e = cudaFuncSetAttribute(k_mlp_tc<MLP_TRAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, MLP_SMEM); attr[2] = e == cudaSuccess; }
+        e = opt_in(2, k_mlp_tc<MLP_TRAIN>);
         if (e == cudaSuccess) k_mlp_tc<MLP_TRAIN><<<grid, MT, MLP_SMEM, s>>>(a);
         break;
     }

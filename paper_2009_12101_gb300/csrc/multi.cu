@@ -28,6 +28,7 @@
 #include <type_traits>
 
 #include "../../include/cbgmres.h"
+#include "cbg_context.h"
 #include "cbg_kernels.cuh"
 #include "cbg_stream.cuh"
 
@@ -321,15 +322,16 @@ __global__ void __launch_bounds__(256) k_multi_sum(const double* part, int nblk,
 template <int FMT, int KP, bool DIRECT> void launch_multi(int grid, cudaStream_t s, const MultiArgs& a)
 {
     using G = MultiGeom<FMT, KP>;
-    static const int stages = [] {
+    static PerContext<int> plan;
+    const int stages = plan.get([](int& st) {
         cudaFuncAttributes fa{};
-        const int st = cudaFuncGetAttributes(&fa, k_dot_multi<FMT, KP, DIRECT>) == cudaSuccess
+        st = cudaFuncGetAttributes(&fa, k_dot_multi<FMT, KP, DIRECT>) == cudaSuccess
                            ? tma_stages(G::STAGE, (int)fa.sharedSizeBytes) : 0;
         if (st >= 2)
             cudaFuncSetAttribute(k_dot_multi<FMT, KP, DIRECT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)tma_smem_bytes(st, G::STAGE));
-        return st;
-    }();
+        return true;
+    });
     k_dot_multi<FMT, KP, DIRECT><<<grid, MU_THREADS, tma_smem_bytes(stages, G::STAGE), s>>>(a, stages);
 }
 

@@ -35,6 +35,7 @@
 #include <cmath>
 
 #include "../../include/cbgmres.h"
+#include "cbg_context.h"
 #include "cbg_kernels.cuh"
 #include "cbg_tma.cuh"
 
@@ -606,11 +607,11 @@ int cbg_tc_multi(int64_t n, int ncols, const void* V, int64_t ld, const double* 
     int* eref = reinterpret_cast<int*>(ws + 256 + (size_t)grid * 4 * 8 * TC_M * sizeof(float2));
     if (fault_out) *fault_out = fault;
     if (cudaMemsetAsync(ws, 0, 16, s) != cudaSuccess) return CBG_ERR_CUDA;
-    static const bool attr = [] {
-        cudaFuncSetAttribute(k_dot_multi_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM);
-        return true;
-    }();
-    (void)attr;
+    static PerContext<bool> attr;
+    attr.get([](bool& ok) {
+        ok = cudaFuncSetAttribute(k_dot_multi_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, TC_SMEM) == cudaSuccess;
+        return ok;
+    });
     TcArgs a{};
     a.V = static_cast<const unsigned short*>(V);
     a.ld = ld;

@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "../../include/cbgmres.h"
+#include "cbg_context.h"
 #include "cbg_launch.h"
 
 using namespace cbg;
@@ -620,29 +621,23 @@ private:
     static constexpr unsigned long long POOL_KEEP = 64ull << 20;
     static int device_pool(cudaMemPool_t* out)
     {
-        constexpr int NDEV = 64;
-        static std::mutex mu;
-        static cudaMemPool_t pools[NDEV] = {};           // per device, created on first use
-        int dev = 0;
-        CBG_CUDA(cudaGetDevice(&dev));
-        if (dev >= NDEV) {
-            CBG_CUDA(cudaDeviceGetDefaultMemPool(out, dev));
-            return CBG_OK;
-        }
-        std::lock_guard<std::mutex> lk(mu);
-        if (!pools[dev]) {
-            cudaMemPoolProps pr{};
-            pr.allocType = cudaMemAllocationTypePinned;
-            pr.location.type = cudaMemLocationTypeDevice;
-            pr.location.id = dev;
-            cudaMemPool_t p = nullptr;
-            unsigned long long keep = POOL_KEEP;
-            CBG_CUDA(cudaMemPoolCreate(&p, &pr));
-            CBG_CUDA(cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep));
-            pools[dev] = p;
-        }
-        *out = pools[dev];
-        return CBG_OK;
+        static PerContext<cudaMemPool_t> pools;          // (a device reset destroys them)
+        int rc = CBG_OK;
+        *out = pools.get([&](cudaMemPool_t& p) {
+            auto make = [&]() -> int {
+                cudaMemPoolProps pr{};
+                pr.allocType = cudaMemAllocationTypePinned;
+                pr.location.type = cudaMemLocationTypeDevice;
+                unsigned long long keep = POOL_KEEP;
+                CBG_CUDA(cudaGetDevice(&pr.location.id));
+                CBG_CUDA(cudaMemPoolCreate(&p, &pr));
+                CBG_CUDA(cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep));
+                return CBG_OK;
+            };
+            rc = make();
+            return rc == CBG_OK;
+        });
+        return rc;
     }
     cudaStream_t s_;
     unsigned char* p_ = nullptr;
