@@ -331,6 +331,17 @@ int cbgmres_spmv_group(const cbg_handle* h);
  * which has no pipelined dot). */
 int cbgmres_test_stall(cbg_handle* h, int dots, long long wait_cycles);
 
+/* The same for the kernels whose blocks wait on one another.  kernel 0: in the next
+ * restart cycle that runs as one launch (small matrices) the last block does not arrive
+ * at barrier number `at` (1, 2, ...: four a step, five with CBG_PC_SPAI and CBG_PC_BJ4;
+ * beyond the cycle's last barrier nothing happens).  kernel 1: in the `at`-th launch of
+ * the kernel that forms w - V h and V^T of it together the last block does not arrive;
+ * the solve then runs the kernels of a step separately.  The waits give up after
+ * wait_cycles clock cycles, the solve returns CBG_ERR_TIMEOUT, and the next solve on h
+ * runs normally.  Errors: CBG_ERR_ARG, CBG_ERR_UNSUPPORTED (the handle does not run that
+ * kernel). */
+int cbgmres_test_withhold(cbg_handle* h, int kernel, int at, long long wait_cycles);
+
 /* Copy the accumulated per-kernel profile of a handle (options.profile == 1) into
  * *out; reset != 0 clears it afterwards.  Errors: CBG_ERR_ARG. */
 int cbgmres_profile(cbg_handle* h, cbg_profile* out, int reset);

@@ -115,6 +115,7 @@ def lib():
             L.cbgmres_spmv.argtypes = [vp, vp, vp]
             L.cbgmres_profile.argtypes = [vp, C.POINTER(Profile), i32]
             L.cbgmres_test_stall.argtypes = [vp, i32, C.c_int64]
+            L.cbgmres_test_withhold.argtypes = [vp, i32, i32, C.c_int64]
             L.cbgmres_spmv_group.argtypes = [vp]
             L.cbgmres_debug_guard_check.argtypes = [vp, i32]
             L.cbgmres_destroy.argtypes = [vp]
@@ -336,6 +337,12 @@ class Solver:
         """Failure-path test: the next `dots` pipelined dot launches withhold their first
         bulk-copy stage and give up their waits after `wait_cycles` clock cycles."""
         _check(lib().cbgmres_test_stall(self._h, int(dots), int(wait_cycles)), "cbgmres_test_stall")
+
+    def test_withhold(self, kernel: str, at: int = 1, wait_cycles: int = 2_000_000):
+        """Failure-path test: one block skips barrier `at` of the next single-launch "cycle", or
+        that of the `at`-th one-pass ("pass") launch; the waits give up after `wait_cycles`."""
+        _check(lib().cbgmres_test_withhold(self._h, {"cycle": 0, "pass": 1}[kernel], int(at), int(wait_cycles)),
+               "cbgmres_test_withhold")
 
     def spmv(self, x):
         torch = _torch()

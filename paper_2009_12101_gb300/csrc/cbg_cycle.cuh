@@ -15,7 +15,7 @@
 // columns, its lanes over the blocks), so that all hold the same coefficients without a
 // further exchange.  The Givens update (a serial FP64 chain of 5-7 us) runs on an extra warp
 // of block 0 while the blocks go on with the next step; its decision to end the cycle is
-// read after the next step's second barrier, so at most one SpMV and two basis products are
+// read after the next step's second barrier, so at most one SpMV and three basis products are
 // computed in vain per cycle.
 //
 // With RES the own rows of the whole basis stay in shared memory as well, and only the
@@ -69,6 +69,7 @@ struct CycleArgs {
     unsigned int* counter;    // arrivals; zero when the launch starts
     int* fault;               // set when a wait ran out
     long long limit;          // clock cycles a wait may take
+    int withhold;             // test of the failure path: the last block does not arrive at this barrier (0: none)
 };
 // their sizes in float2 (8 bytes); norm starts on a 16-byte boundary
 constexpr size_t CY_PART = (size_t)2 * MAXCOLS * CY_MAXG, CY_NORM = (size_t)4 * CY_MAXG, CY_WMAX = CY_MAXG, CY_COEF = (size_t)4 * MAXCOLS;
@@ -105,14 +106,16 @@ __device__ __forceinline__ void cy_take(int id) { asm volatile("bar.sync %0, %1;
 
 // Barrier of the compute warps of all blocks: thread 0 releases the block's writes into a
 // counter that only grows within the launch and waits (bounded) until every block has
-// arrived as often as this one.  Sets sm.fail when the wait ran out.
-__device__ __forceinline__ void cy_grid_sync(const CycleArgs& a, CycleShared& sm, unsigned& epoch)
+// arrived as often as this one.  Sets sm.fail when the wait ran out.  skip: the epoch at which the
+// block does not arrive (a test; 0: it always does).
+__device__ __forceinline__ void cy_grid_sync(const CycleArgs& a, CycleShared& sm, unsigned& epoch, unsigned skip)
 {
     epoch += gridDim.x;
     cy_sync();
     if (threadIdx.x == 0) {
         unsigned now;
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counter) : "memory");
+        if (epoch != skip)
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.counter) : "memory");
         const long long t0 = clock64();
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(now) : "l"(a.counter) : "memory");
@@ -673,6 +676,8 @@ template <int FMT, bool RES> struct Cycle {
         const long long vstride = RES ? (long long)a.rows * BS : a.ldb;
         float2* part2 = a.part + MAXCOLS * CY_MAXG;
         unsigned epoch = 0;
+        const unsigned skip = blockIdx.x + 1 == gridDim.x ? a.withhold * gridDim.x : 0u;
+        bool open = false;                        // block 0: the Givens warp will arrive at barrier 3
         volatile int* fail = &sm.fail;
         if (t == 0) sm.scale[0] = a.d.scales[0];
         for (int r = t; r < R; r += CY_CT) wh[r] = wl[r] = 0.f;
@@ -690,7 +695,7 @@ template <int FMT, bool RES> struct Cycle {
             // w = A M^{-1} v_j, omega
             if (a.prow) {
                 precondition(a, vj, sm.scale[j], r0, R);
-                cy_grid_sync(a, sm, epoch);
+                cy_grid_sync(a, sm, epoch, skip);
                 if (*fail) break;
                 spmv<-1>(a, sm, a.z, 1.0, r0, R, wh, wl);
             } else {
@@ -699,25 +704,29 @@ template <int FMT, bool RES> struct Cycle {
             cy_sync();
             // h = V^T w
             dot(a, sm, red, vs, vstride, R, ncols, wh, wl, a.part, true);
-            cy_grid_sync(a, sm, epoch);
+            cy_grid_sync(a, sm, epoch, skip);
             if (*fail) break;
             collect(a, sm, a.part, ncols, hj);
             // w1 = w - V h ; u = V^T w1
             axpy<false>(a, sm, vs, vstride, r0, R, ncols, wh, wl, split);
             dot(a, sm, red, vs, vstride, R, ncols, wh, wl, part2, false);
-            if (b == 0 && j > 0) cy_take(3);                          // the Givens update of step j - 1
-            cy_grid_sync(a, sm, epoch);
+            if (b == 0 && j > 0) {
+                cy_take(3);                                           // the Givens update of step j - 1
+                open = false;
+            }
+            cy_grid_sync(a, sm, epoch, skip);
             if (*fail || (j > 0 && *(volatile int*)&a.d.st->active == 0)) break;
             collect(a, sm, part2, ncols, hj + MAXCOLS);
             // w2 = w1 - V u, its norms
             axpy<true>(a, sm, vs, vstride, r0, R, ncols, wh, wl, split);
             put_norms(a, sm);
-            cy_grid_sync(a, sm, epoch);
+            cy_grid_sync(a, sm, epoch, skip);
             if (*fail) break;
             collect_norms(a, sm, ncols, &sm.omega[j & 1]);
             if (b == 0) {
                 if (t == 0) a.d.scales[ncols] = sm.ep.scale;
                 cy_post(2);                                           // column j to the Givens warp
+                open = j + 1 < kcap;
             }
             // v_{j+1}
             {
@@ -735,7 +744,7 @@ template <int FMT, bool RES> struct Cycle {
                     }
                 }
             }
-            if (j + 1 < kcap) cy_grid_sync(a, sm, epoch);
+            if (j + 1 < kcap) cy_grid_sync(a, sm, epoch, skip);
             if (*fail) break;
         }
         if (*fail) {
@@ -743,9 +752,13 @@ template <int FMT, bool RES> struct Cycle {
                 record_fault(nullptr, a.fault);
                 sm.quit = 1;
             }
-            if (b == 0) {                                             // release the Givens warp
+            if (b == 0) {
+                // release the Givens warp: once it has done with the column it was given (a second
+                // arrival at barrier 2 before it took the first would be one too many) it waits
+                // there for the next one, unless it has ended the cycle
+                if (open) cy_take(3);
                 cy_sync();
-                cy_post(2);
+                if (*(volatile int*)&a.d.st->active != 0) cy_post(2);
             }
         }
     }

@@ -237,9 +237,10 @@ struct DotArgs {
     double* out;              // [ncols]
     const int* active;        // skip when *active == 0 (may be null)
     const float* wdf;         // w split into FP32 pairs, planar: hi[nrows] then lo[nrows] (DF32; may be null)
-    // pipelined dot only: waits give up after wait_limit clock cycles (0: the default of
-    // about a second); withhold != 0 makes the producer skip its first work item (no
-    // arrival, no copies), so that the waits on it run out -- a test of the timeout path
+    // pipelined dot and one-pass kernel: waits give up after wait_limit clock cycles (0: the
+    // default of about a second); withhold != 0 makes the dot's producer skip its first work
+    // item (no arrival, no copies) and the one-pass kernel's last block the grid barrier, so that
+    // the waits on them run out -- a test of the timeout path
     long long wait_limit;
     int withhold;
 };

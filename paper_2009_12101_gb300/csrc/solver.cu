@@ -113,6 +113,7 @@ const Ops& ops_for(int fmt)
 
 long long round_up(long long a, long long b) { return (a + b - 1) / b * b; }
 
+constexpr int CNT_WORDS = 16;                     // DevArrays::counters
 constexpr int CNT_CYCLE = 8;                      // DevArrays::counters slot of the single-launch cycle
 constexpr long long SPMV_TUNE_MIN_ROWS = 65536;   // create times the SpMV schedules from here on
 
@@ -476,6 +477,8 @@ struct cbg_handle {
     bool use_sell = false;
     int grid_sell = 0;
     int test_stall = 0;            // cbgmres_test_stall: pipelined dots still to be stalled
+    int test_cycle = 0;            // cbgmres_test_withhold: barrier of the next single-launch cycle,
+    int test_pass = 0;             // one-pass launches up to the one that is to fail
     long long test_wait = 0;       //   and their wait limit in clock cycles
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     std::vector<cudaEvent_t> step_ev;
@@ -822,6 +825,11 @@ void enqueue_cycle(cbg_handle* h)
     a.counter = h->d.counters + CNT_CYCLE;
     a.fault = &h->d.st->fault;
     a.limit = WAIT_LIMIT_CYCLES;
+    if (h->test_cycle > 0) {                  // cbgmres_test_withhold: this launch times out
+        a.withhold = h->test_cycle;
+        a.limit = h->test_wait;
+        h->test_cycle = 0;
+    }
     launch(h, 4, 0.0, [&] {
         ops_for(h->fmt).cycle(h->cycle_resident, h->cycle_grid, h->cycle_smem, h->stream, a);
     });
@@ -1046,6 +1054,13 @@ void enqueue_step(cbg_handle* h, int j)
                 pa.d = da;
                 pa.coef = h->d.h;
                 pa.wdf = wdf;
+                if (h->test_pass != 0) {      // cbgmres_test_withhold; -1: the barrier word is one
+                    if (h->test_pass > 0 && --h->test_pass == 0) {   // arrival short from here on
+                        pa.d.withhold = 1;
+                        h->test_pass = -1;
+                    }
+                    pa.d.wait_limit = h->test_wait;
+                }
                 launch(h, 1, pass_bytes, [&] { op.pass(h->grid_tma, s, pa, &h->d.st->fault); });
             } else {
                 launch(h, 0, pass_bytes, run_dot);
@@ -1143,7 +1158,11 @@ int read_state(cbg_handle* h, DevState* out)
 #endif
         return CBG_ERR_ARG;
     }
-    if (out->fault) return CBG_ERR_TIMEOUT;   // a pipelined kernel stopped waiting
+    if (out->fault) {                          // a kernel stopped waiting: its barrier words start over
+        CBG_CUDA(cudaMemsetAsync(h->d.counters, 0, CNT_WORDS * sizeof(unsigned int), h->stream));
+        h->test_pass = 0;
+        return CBG_ERR_TIMEOUT;
+    }
     return CBG_OK;
 }
 
@@ -1237,8 +1256,8 @@ int run_solve(cbg_handle* h, const double* b, double* x, double tol, long long m
             cycles++;
             nvtxRangePushA("cbgmres cycle");
             enqueue_first_vector(h);
-            // (a requested stall of the pipelined dot needs the stepwise kernels)
-            const bool single = h->cycle_grid > 0 && h->test_stall == 0;
+            // (a requested stall of the pipelined dot or of the pass needs the stepwise kernels)
+            const bool single = h->cycle_grid > 0 && h->test_stall == 0 && h->test_pass == 0;
             if (single) enqueue_cycle(h);
             const int kcap = single ? 0 : hs.kcap;
             for (int j = 0; j < kcap; j++) {
@@ -1515,7 +1534,7 @@ int cbgmres_create(const cbg_csr* A, int restart, int fmt, const cbg_options* op
     size_t o_part = take(sizeof(double) * (size_t)h->gridmax * MAXCOLS);
     size_t o_pn = take(sizeof(double) * (size_t)h->gridmax * 4);
     size_t o_ps = take(sizeof(double) * (size_t)h->gridmax * 2);
-    size_t o_cnt = take(sizeof(unsigned int) * 16);
+    size_t o_cnt = take(sizeof(unsigned int) * CNT_WORDS);
     // one launch per restart cycle: the default arithmetic and orthogonalisation; profiling
     // times the kernels of a step, so it keeps them apart
     const bool single = o.arith == CBG_ARITH_DF32 && o.ortho == CBG_ORTHO_CGS && o.reorth == CBG_REORTH_ALWAYS &&
@@ -1777,6 +1796,17 @@ int cbgmres_test_stall(cbg_handle* h, int dots, long long wait_cycles)
     if (!h || dots < 0 || wait_cycles < 1) return CBG_ERR_ARG;
     if (!h->use_tma) return CBG_ERR_UNSUPPORTED;
     h->test_stall = dots;
+    h->test_wait = wait_cycles;
+    return CBG_OK;
+}
+
+int cbgmres_test_withhold(cbg_handle* h, int kernel, int at, long long wait_cycles)
+{
+    if (!h || (kernel != 0 && kernel != 1) || at < 1 || wait_cycles < 1) return CBG_ERR_ARG;
+    if (kernel == 0 ? h->cycle_grid == 0 : !(h->use_tma && h->opt.ortho == CBG_ORTHO_CGS && h->opt.reorth == CBG_REORTH_ALWAYS))
+        return CBG_ERR_UNSUPPORTED;
+    h->test_cycle = kernel == 0 ? at : 0;
+    h->test_pass = kernel == 1 ? at : 0;
     h->test_wait = wait_cycles;
     return CBG_OK;
 }
