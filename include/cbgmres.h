@@ -264,7 +264,9 @@ int cbg_decode(int fmt, int64_t n, const void* codes, double scale, double* out,
                void* stream);
 
 /* ---- basis products, exposed for parity checks (CGS and re-orthogonalisation, Fig. 1) ---
- * V: device codes, ncols columns of leading dimension ld elements; scales[ncols] host.
+ * V: device codes, ncols columns of leading dimension ld elements, on a 16-byte boundary
+ * (else CBG_ERR_ARG; w too with CBG_ARITH_FP64 and in cbg_basis_dot_noalloc);
+ * scales[ncols] host.
  * cbg_basis_dot:  h[k] = sum_i dec(V[i,k]) w[i]      (h: host, w: device)
  * cbg_basis_axpy: w[i] -= sum_k dec(V[i,k]) h[k]     (h: host, w: device, in place)
  * arith: cbg_arith.  Synchronise `stream`. */
@@ -287,7 +289,8 @@ int cbg_basis_axpy(int fmt, int arith, int64_t n, int ncols, const void* V, int6
  *   workspace: device scratch of at least cbg_basis_dot_multi_workspace(ld, ncols, k)
  *      bytes, owned by the caller, not shared between concurrent calls.
  * Asynchronous on `stream` (no allocation, no synchronisation).  Errors: CBG_ERR_ARG
- * (sizes, null pointers, workspace too small), CBG_ERR_CUDA. */
+ * (sizes, null pointers, workspace too small, a pointer not aligned to its type),
+ * CBG_ERR_CUDA. */
 size_t cbg_basis_dot_multi_workspace(int64_t ld, int ncols, int k);
 int cbg_basis_dot_multi(int fmt, int64_t n, int ncols, const void* V, int64_t ld, const double* scales, int k,
                         const double* W, int64_t ldw, double* H, void* workspace, size_t ws_bytes,

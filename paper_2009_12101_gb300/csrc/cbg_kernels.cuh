@@ -19,6 +19,7 @@ constexpr int THREADS = 256;
 constexpr int TILE_ROWS = 4096;      // ld (padded rows) is a multiple of this
 constexpr int MAXCOLS = 320;         // largest restart length + 1 supported by the kernels
 constexpr int DOT_MIN_ROWS = 1024;   // the dot kernel's grid gives every block >= this many rows
+inline bool aligned(const void* p, size_t bytes) { return reinterpret_cast<size_t>(p) % bytes == 0; }
 constexpr int ARITH_DF32 = 0;
 constexpr int ARITH_FP64 = 1;
 

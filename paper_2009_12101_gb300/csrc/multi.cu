@@ -51,8 +51,6 @@ constexpr int MU_CG = MU_CS * MU_CPW;   // columns per stage
 constexpr int MU_THREADS = (MU_CW + 1) * 32;
 constexpr int MU_CHAIN = 32;         // rows a lane accumulates before its sums are folded (one pair of vectors: half)
 
-__host__ __device__ inline bool aligned16(const void* p) { return (reinterpret_cast<size_t>(p) & 15) == 0; }
-
 template <int FMT, int KP> struct MultiGeom {
     static constexpr int BS = FmtInfo<FMT>::bytes;
     static constexpr int E = 16 / BS;                       // rows per lane
@@ -337,7 +335,7 @@ template <int FMT, int KP, bool DIRECT> void launch_multi(int grid, cudaStream_t
 
 template <int FMT, int KP> void launch_multi(int grid, cudaStream_t s, const MultiArgs& a)
 {
-    if (aligned16(a.V)) launch_multi<FMT, KP, false>(grid, s, a);
+    if (aligned(a.V, 16)) launch_multi<FMT, KP, false>(grid, s, a);
     else launch_multi<FMT, KP, true>(grid, s, a);
 }
 
@@ -423,8 +421,10 @@ int cbg_basis_dot_multi_path(int fmt, int64_t n, int ncols, const void* V, int64
         ld < n || ld % TILE_ROWS || !scales || !W || ldw < n || !H || !workspace ||
         ws_bytes < cbg_basis_dot_multi_workspace(ld, ncols, k) || path < 0 || path > 2)
         return CBG_ERR_ARG;
+    if (!aligned(V, cbgmres_format_bytes(fmt)) || !aligned(W, 8) || !aligned(scales, 8) || !aligned(H, 8))
+        return CBG_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const bool tc_ok = fmt == CBG_F16 && ncols <= 128 && aligned16(V);   // (it reads 16 bytes at a time)
+    const bool tc_ok = fmt == CBG_F16 && ncols <= 128 && aligned(V, 16);   // (it reads 16 bytes at a time)
     if (path == 2 && !tc_ok) return CBG_ERR_UNSUPPORTED;
     const bool tc = path == 2 || (path == 0 && tc_ok);
     // groups of up to KMAX vectors, one after the other on the stream (the workspace is reused)

@@ -82,6 +82,7 @@ extern "C" int cbg_basis_dot_noalloc(int fmt, int arith, int64_t n, int ncols, c
         ncols < 1 || !V || ld < n || ld % TILE_ROWS || !scales || !w || !h)
         return CBG_ERR_ARG;
     if (ncols > NOALLOC_MAX_COLS) return CBG_ERR_ARG;   // beyond the static scratch
+    if (!aligned(V, 16) || !aligned(w, 16)) return CBG_ERR_ARG;   // both are read 16 bytes at a time
     double* base = nullptr;
     int rc = scratch_for_current_device(&base);
     if (rc) return rc;

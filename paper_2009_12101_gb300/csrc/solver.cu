@@ -1931,6 +1931,8 @@ int cbg_basis_dot(int fmt, int arith, int64_t n, int ncols, const void* V, int64
     if (fmt_bytes(fmt) == 0 || (arith != 0 && arith != 1) || n < 1 || ncols < 1 || ncols > MAXCOLS || !V ||
         ld < n || ld % TILE_ROWS || !scales || !w || !hout)
         return CBG_ERR_ARG;
+    // 16-byte accesses: the codes, and w in FP64 arithmetic (DF32 splits it element by element)
+    if (!aligned(V, 16) || !aligned(w, arith == CBG_ARITH_FP64 ? 16 : 8)) return CBG_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const Ops& op = ops_for(fmt);
     const bool tma = arith == CBG_ARITH_DF32;
@@ -1984,6 +1986,7 @@ int cbg_basis_axpy(int fmt, int arith, int64_t n, int ncols, const void* V, int6
     if (fmt_bytes(fmt) == 0 || (arith != 0 && arith != 1) || n < 1 || ncols < 1 || ncols > MAXCOLS || !V ||
         ld < n || ld % TILE_ROWS || !scales || !hcoef || !w)
         return CBG_ERR_ARG;
+    if (!aligned(V, 16) || !aligned(w, 8)) return CBG_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     const Ops& op = ops_for(fmt);
     const long long blocks = ld / ((long long)THREADS * (16 / fmt_bytes(fmt)));
