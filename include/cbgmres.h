@@ -397,8 +397,8 @@ int cbgmres_solve_batched(cbg_batch* bt, const double* b, double* x, double tol,
  * problem (x restored to x0 before each trial) with a thread per SpMV row, then the
  * SpMV's lanes per row (2, 4, 8: the lanes of a row split its nonzeros) for the best of
  * them, and keep the fastest; cache_path (may be NULL) is a JSON-lines file consulted
- * first and appended to, keyed by GPU, format, restart length, system count and total
- * rows.  The chosen cluster size and split threshold are returned
+ * first and appended to, keyed by GPU, format, restart length, system count, total rows
+ * and the kernels' version (timings of older kernels are not used).  The chosen cluster size and split threshold are returned
  * (cbgmres_batched_spmv_lanes(bt, 0) reports the lanes). */
 int cbgmres_tune_batched(cbg_batch* bt, const double* b, double* x, double tol, int64_t maxit,
                          const char* cache_path, int* cluster_out, int* split_rows_out);

@@ -329,6 +329,10 @@ int run_graph(cbg_batch* bt, double tol, long long maxit)
     return CBG_OK;
 }
 
+// Raised when the batched kernel changes enough for old timings to mislead: schedules that were
+// cached for other kernels are not taken.
+constexpr int TUNE_VERSION = 2;
+
 std::string tune_key(const cbg_batch* bt)
 {
     cudaDeviceProp p{};
@@ -337,7 +341,7 @@ std::string tune_key(const cbg_batch* bt)
     cudaGetDeviceProperties(&p, dev);
     std::ostringstream os;
     os << p.name << "|sm" << p.major << p.minor << "|fmt" << bt->fmt << "|m" << bt->m << "|nsys" << bt->nsys
-       << "|rows" << bt->total_rows << "|maxn" << bt->max_n;
+       << "|rows" << bt->total_rows << "|maxn" << bt->max_n << "|k" << TUNE_VERSION;
     return os.str();
 }
 
