@@ -171,7 +171,8 @@ typedef struct {
     double true_relres;      /* ||b - A x||_2 / ||b||_2 at exit (FP64, explicit)       */
     double est_relres;       /* last recurrence residual |g_{j+1}| / ||b||_2           */
     double ms_total;         /* wall time of the solve on the stream (CUDA events)     */
-    double bytes_model;      /* model HBM bytes: SpMV + 4 basis passes per step         */
+    double bytes_model;      /* model HBM bytes: SpMV + 4 basis passes per step, 3 where one
+                                kernel forms w - V h and V^T of it                     */
     int32_t status;          /* same value as the function's return                    */
     int32_t fmt_final;       /* basis format of the last cycle (differs from the handle's
                                 only with options.adapt)                                */

@@ -920,6 +920,14 @@ void enqueue_mgs(cbg_handle* h, int j, bool reorth, float* wdf, DotArgs& da, Axp
     }
 }
 
+// Whether a step with ncols columns forms w - V h and V^T of it in one pass over the basis: DF32,
+// CGS with the second pass always, as long as a tile of all columns fits (112 columns)
+bool one_pass(const cbg_handle* h, int ncols)
+{
+    return h->use_tma && h->opt.ortho == CBG_ORTHO_CGS && h->opt.reorth == CBG_REORTH_ALWAYS &&
+           ops_for(h->fmt).pass_fits(ncols);
+}
+
 void enqueue_step(cbg_handle* h, int j)
 {
     const Ops& op = ops_for(h->fmt);
@@ -1037,9 +1045,8 @@ void enqueue_step(cbg_handle* h, int j)
             xa.reorth_flag = &h->d.st->reorth_now;
             xa.eta = h->opt.eta;
         }
-        // DF32, second pass always: this subtraction and the second projection in one pass over
-        // the basis, as long as a tile of all columns fits (112 columns)
-        const bool fused = planes_only && h->use_tma && op.pass_fits(ncols);
+        // this subtraction and the second projection in one pass over the basis
+        const bool fused = one_pass(h, ncols);
         if (!fused) launch(h, 1, pass_bytes, [&] { run_axpy(xa); });
         if (reorth) {
             // re-orthogonalisation: u = V^T w1 ; w2 = w1 - V u ; (h += u in the store kernel);
@@ -1225,15 +1232,17 @@ int run_solve(cbg_handle* h, const double* b, double* x, double tol, long long m
         const int L = (int)h->step_ev.size();
         long long iters_before = -1;
         double prev_beta = INFINITY;
-        bool stagnated = false;
+        bool stagnated = false, single = false;     // (single: the last cycle ran as one launch)
         for (;;) {
             enqueue_residual(h, b, x);
             launch(h, 4, 0.0, [&] { k_cycle_start<<<1, 1, 0, s>>>(h->d, maxit_eff, h->m); });
             int rc = read_state(h, &hs);
             if (rc) return rc;
             harvest_profile(h);
-            for (int j = 0; j < hs.last_k; j++)
-                bytes += spmv_bytes + 4.0 * (double)(j + 1) * (double)h->n * (double)fmt_bytes(h->fmt);
+            for (int j = 0; j < hs.last_k; j++) {
+                const double passes = !single && one_pass(h, j + 1) ? 3.0 : 4.0;
+                bytes += spmv_bytes + passes * (double)(j + 1) * (double)h->n * (double)fmt_bytes(h->fmt);
+            }
             if (!hs.active) break;
             if (k_only > 0 && cycles >= 1) break;
             if (cycles > 0 && hs.iters == iters_before) return CBG_ERR_CUDA;   // no progress: device work failed
@@ -1257,7 +1266,7 @@ int run_solve(cbg_handle* h, const double* b, double* x, double tol, long long m
             nvtxRangePushA("cbgmres cycle");
             enqueue_first_vector(h);
             // (a requested stall of the pipelined dot or of the pass needs the stepwise kernels)
-            const bool single = h->cycle_grid > 0 && h->test_stall == 0 && h->test_pass == 0;
+            single = h->cycle_grid > 0 && h->test_stall == 0 && h->test_pass == 0;
             if (single) enqueue_cycle(h);
             const int kcap = single ? 0 : hs.kcap;
             for (int j = 0; j < kcap; j++) {
