@@ -639,6 +639,13 @@ template <int FMT> struct BatchedSolver {
         __syncthreads();
     }
 
+    // e with omega < 2^e, within the float exponents; 0 for zero and what is not finite
+    static __device__ __forceinline__ int norm_exponent(double omega)
+    {
+        const int e = ((__double2hiint(omega) >> 20) & 0x7FF) - 1022;
+        return e == -1022 || e == 1025 ? 0 : max(-126, min(126, e));
+    }
+
     // w -= V coef over own rows; with NORMS, also the block's sum of squares (triples of floats,
     // tf_add, into sm->red[0]) and, for the formats whose scale needs it, the maximum of |w| (into
     // sm->red[1]).  Blocks with fewer row chunks than threads split the columns over the
@@ -667,6 +674,10 @@ template <int FMT> struct BatchedSolver {
         const int ks = 1 << lk, cpw = 32 >> lk, mk = lane >> (5 - lk), mch = lane & (cpw - 1);
         float4 ss = make_float4(0.f, 0.f, 0.f, 0.f);
         float2 mx = make_float2(0.f, 0.f);
+        // the squares are taken of w 2^-e with omega < 2^e: an operator whose largest value is so small
+        // that it could not be normalised would have them underflow in FP32
+        const int e = NORMS ? norm_exponent(sm->omega) : 0;
+        const float down = __int_as_float((127 - e) << 23);
         for (int base = warp * cpw; base < nch; base += NW * cpw) {
             const int ch = base + mch;
             const bool in = ch < nch;
@@ -727,11 +738,12 @@ template <int FMT> struct BatchedSolver {
                     wl[r] = l;
                     if constexpr (NORMS) {
                         // h^2 = p + q and 2 h l = t + u exactly, l^2
-                        const float p = __fmul_rn(h, h), q = __fmaf_rn(h, h, -p);
-                        const float h2 = __fadd_rn(h, h), t = __fmul_rn(h2, l), u = __fmaf_rn(h2, l, -t);
+                        const float hs = __fmul_rn(h, down), ls = __fmul_rn(l, down);
+                        const float p = __fmul_rn(hs, hs), q = __fmaf_rn(hs, hs, -p);
+                        const float h2 = __fadd_rn(hs, hs), t = __fmul_rn(h2, ls), u = __fmaf_rn(h2, ls, -t);
                         float y, z;
                         two_sum(t, q, y, z);
-                        tf_add(ss, p, y, __fadd_rn(z, __fmaf_rn(l, l, u)));
+                        tf_add(ss, p, y, __fadd_rn(z, __fmaf_rn(ls, ls, u)));
                         if constexpr (SCALED) {
                             const float ah = fabsf(h), al = h < 0.f ? -l : l;
                             if (!(ah < mx.x || (ah == mx.x && al <= mx.y))) mx = make_float2(ah, al);
@@ -761,7 +773,7 @@ template <int FMT> struct BatchedSolver {
                     tf_add(t, wsum[w]);
                     if (!(wmax[w].x < m.x || (wmax[w].x == m.x && wmax[w].y <= m.y))) m = wmax[w];
                 }
-                sm->red[0] = tf_to_double<true>(t);
+                sm->red[0] = __dmul_rn(tf_to_double<true>(t), pow2d(2 * e));
                 sm->red[1] = df_to_double(m.x, m.y);
             }
         }
@@ -821,9 +833,8 @@ template <int FMT> struct BatchedSolver {
             const double rr = hypot(r0v, hnt);
             double c = 1.0, sn = 0.0;
             if (rr != 0.0) {
-                const double ri = 1.0 / rr;
-                c = __dmul_rn(r0v, ri);
-                sn = __dmul_rn(hnt, ri);
+                c = r0v / rr;                                  // (1 / rr overflows for a subnormal rr)
+                sn = hnt / rr;
             }
             sm->cs[j] = c;
             sm->sn[j] = sn;
