@@ -81,9 +81,12 @@ typedef enum { CBG_ORTHO_CGS = 0, CBG_ORTHO_MGS = 1 } cbg_ortho;
  *   the error bounds of the basis products and of the SpMV rows are those of FP64 with
  *   the unit roundoff 2^-46 in place of 2^-53: 2^6 - 2^8 looser than the same sums in
  *   native FP64, 2^20 tighter than FP32.  The basis dot sums each thread's chain of
- *   about n / 38,912 products in double-float and the chains in FP64, so its bound,
- *   about (n / 38,912) 2^-46 sum |v_i w_i|, stays below FP64's recursive-summation
- *   bound n 2^-53 sum |v_i w_i| for every n >= 128.  The per-step SpMV forms each
+ *   about n / 38,912 products and its warp in double-float and the warps and blocks in
+ *   FP64, so its bound, about (n / 38,912 + 5) 2^-46 sum |v_i w_i|, stays below FP64's
+ *   recursive-summation bound n 2^-53 sum |v_i w_i| for every n >= 1024.  Where a restart
+ *   cycle runs as one launch (small matrices) the chains, of n / 77,824 products, are
+ *   summed in double-float over the blocks too (some 20 additions more); the second
+ *   Gram-Schmidt pass takes in what the first one's sums missed.  The per-step SpMV forms each
  *   product val * x exactly as an FP32 pair from the values split once into FP32 hi / lo
  *   planes (a relative 2^-48 perturbation of A) and delivers w as such planes.  The
  *   per-step operator (A, or A D^{-1} under Jacobi) is normalised by a power of two so
@@ -96,8 +99,9 @@ typedef enum { CBG_ORTHO_CGS = 0, CBG_ORTHO_MGS = 1 } cbg_ortho;
  * CBG_ARITH_FP64: every product and sum is a native FP64 operation, as the paper
  *   prescribes; on GB300 the basis products then run at FP64-pipe speed.
  * With CBG_ARITH_DF32 the norms of the Arnoldi step (omega = ||A v_j|| in the SpMV,
- * ||w|| in the last CGS pass) are also summed in double-float per thread and combined
- * in FP64.  The residual SpMV (b - Ax, which decides convergence), ||r||, the Givens
+ * ||w|| in the last CGS pass) are also summed in double-float per thread, and across
+ * threads and blocks to FP64's precision or better (triples of floats).  The residual
+ * SpMV (b - Ax, which decides convergence), ||r||, the Givens
  * rotations, the least-squares solve and the solution update are FP64 in both modes. */
 typedef enum { CBG_ARITH_DF32 = 0, CBG_ARITH_FP64 = 1 } cbg_arith;
 

@@ -25,8 +25,8 @@
 // splits and epilogues; only the order of the sums differs, and the columns' sums over blocks are
 // of double-float pairs (see collect).
 //
-// What bounds it: 64^2 f64, restart 100, takes 18 us per step (72 us as separate kernels): 11.5k
-// of 36k cycles in the four barriers (about 1.4 us each: one release, one poll), 6k in the
+// What bounds it: 64^2 f64, restart 100, takes 18.5 us per step (72 us as separate kernels): 11.5k
+// of 37k cycles in the four barriers (about 1.4 us each: one release, one poll), 6k in the
 // two sums over the blocks (an L2 round trip and a warp tree each), 11k in the basis
 // products, 3.6k in the SpMV's chain of three loads, 3k in the FP64 root and division of
 // the norm and the encoding.  Tagged exchange words in place of barriers were slower: every

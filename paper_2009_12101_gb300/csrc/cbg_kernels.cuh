@@ -3,8 +3,9 @@
 //
 // Data layout in HBM (per solver handle):
 //   V       (m+1) columns of codes, column k at V + k*ldb, ldb = ld * bytes(fmt),
-//           ld = n rounded up to TILE_ROWS; rows n..ld-1 are zero and stay zero, so every
-//           kernel processes whole tiles without bounds checks on the basis.
+//           ld = n rounded up to TILE_ROWS; rows n..ld-1 are zero and stay zero (a change of
+//           format, which moves the columns, clears them), so every kernel processes whole
+//           tiles without bounds checks on the basis.
 //   scales  (m+1) FP64 decode factors (sigma_k, 2^e_k or 1)
 //   vectors FP64 arrays of ld elements, zero padded.
 #pragma once

@@ -1,11 +1,11 @@
 // noalloc.cu -- basis dot product h = V^T w that allocates no device memory.
 //
-// cbg_basis_dot allocates its scratch (per-block partial sums, the last-block counter,
-// device copies of the scales and of the result) with cudaMalloc and frees it with
-// cudaFree on every call.  Some callers cannot do that: an application whose device
-// memory is owned by another allocator (a framework's caching allocator or a
-// pre-sized pool) may have no memory left for a library's private cudaMalloc, and a
-// latency-critical loop cannot afford cudaFree, which synchronises the whole device.
+// cbg_basis_dot takes its scratch (per-block partial sums, the barrier word, device copies
+// of the scales and of the result) from a stream-ordered pool of the library's own, which
+// keeps up to 64 MiB.  Some callers cannot have that: an application whose device memory is
+// owned by another allocator (a framework's caching allocator or a pre-sized pool) may have
+// no memory left for a library's private allocations, and a call that finds the pool empty
+// waits for the driver to map memory.
 // cbg_basis_dot_noalloc takes the same arguments and keeps its scratch in one
 // file-scope device array instead.  Every GPU that loads this library holds that array
 // (NOALLOC_SCRATCH_BYTES, about 765 KiB) until the process exits.

@@ -763,7 +763,9 @@ int change_format(cbg_handle* h, int fmt)
 // 5.5 -> 4.7, 6.7 -> 7.2.  The single launch reads the basis four times a step out of L2, the
 // stepwise kernels three times with more bytes in flight and more warps in the SpMV: hence
 // limits on the basis's bytes (about the L2 for f64; the 4-byte formats' shares on chip reach
-// further), the rows and the nonzeros.
+// further), the rows and the nonzeros.  The formats of 4 bytes and fewer share one limit: at
+// 88^3 f32, i32 and i16 lose by 1 to 5 % in one launch, f16 alone would gain 4 %.  (The norms'
+// triples of floats, later, cost 0.4 us of a step in the one and 0 to 1 us in the other.)
 bool cycle_worthwhile(long long n, long long nnz, int m, int fmt)
 {
     const double basis = (double)n * (double)(m + 1) * (double)fmt_bytes(fmt);

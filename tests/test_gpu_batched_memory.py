@@ -29,6 +29,7 @@ def test_no_room_for_the_sliced_ell_copy(fmt):
             return used, x.cpu().numpy()
 
     x0 = torch.zeros_like(b)
+    torch.cuda.empty_cache()                             # (nothing is given back under pressure later)
     free = torch.cuda.mem_get_info()[0]
     solve()                                              # (kernels loaded)
     torch.cuda.synchronize()
