@@ -833,8 +833,13 @@ template <int FMT> struct BatchedSolver {
             const double rr = hypot(r0v, hnt);
             double c = 1.0, sn = 0.0;
             if (rr != 0.0) {
-                c = r0v / rr;                                  // (1 / rr overflows for a subnormal rr)
-                sn = hnt / rr;
+                const double ri = 1.0 / rr;
+                c = __dmul_rn(r0v, ri);
+                sn = __dmul_rn(hnt, ri);
+                if (!isfinite(ri)) {                           // a subnormal rr
+                    c = r0v / rr;
+                    sn = hnt / rr;
+                }
             }
             sm->cs[j] = c;
             sm->sn[j] = sn;
